@@ -228,6 +228,8 @@ enum : int { kPtrHost = 0, kPtrHere = 1, kPtrOther = -1 };
 int ptr_where(const void* p, int device);
 int ctx_fail(void* ctx, int code, const char* msg);
 void ctx_count_launches(void* ctx, int n);
+// Owning seat of a loaded policy (-1: shared); id in [0, n_pol).
+int ctx_policy_seat(const void* ctx, int32_t id);
 // Device work space owned by the context, grown on its stream (cudaMallocAsync).
 int ctx_scratch(void* ctx, int64_t bytes, void** out);
 

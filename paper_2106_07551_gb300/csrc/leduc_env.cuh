@@ -1,5 +1,6 @@
 // Leduc hold'em rules on the device (registers only), shared by the fp32 and
-// tensor-core evaluation kernels.
+// tensor-core evaluation kernels; the betting rules are also usable at compile
+// time (the exploitability kernels' betting tree is a constant).
 #pragma once
 
 #include "device_common.cuh"
@@ -13,8 +14,8 @@ namespace malib {
 struct LeducHand {
     int c0, c1, pub;
     int round, con0, con1, raises, nact, actor, done, payoff;
-    __device__ int con_of(int seat) const { return seat ? con1 : con0; }
-    __device__ int card_of(int seat) const { return seat ? c1 : c0; }
+    __host__ __device__ constexpr int con_of(int seat) const { return seat ? con1 : con0; }
+    __host__ __device__ constexpr int card_of(int seat) const { return seat ? c1 : c0; }
 };
 
 __device__ __forceinline__ void leduc_deal(LeducHand& h, uint64_t g, uint64_t seed) {
@@ -31,7 +32,7 @@ __device__ __forceinline__ void leduc_deal(LeducHand& h, uint64_t g, uint64_t se
     h.actor = 0; h.done = 0; h.payoff = 0;
 }
 
-__device__ __forceinline__ unsigned leduc_legal(const LeducHand& h) {
+__host__ __device__ constexpr __forceinline__ unsigned leduc_legal(const LeducHand& h) {
     const int me = h.actor;
     return (h.con_of(1 - me) > h.con_of(me) ? 1u : 0u) | 2u | (h.raises < 2 ? 4u : 0u);
 }
@@ -56,16 +57,16 @@ __device__ __forceinline__ void leduc_obs(const LeducHand& h, float (&o)[17]) {
     o[16] = (lg & 4u) ? 1.f : 0.f;
 }
 
-__device__ __forceinline__ int leduc_showdown(const LeducHand& h) {
+__host__ __device__ constexpr __forceinline__ int leduc_showdown(const LeducHand& h) {
     const int r0 = h.c0 >> 1, r1 = h.c1 >> 1, rp = h.pub >> 1;
-    int w;
+    int w = 0;
     if (r0 == rp) w = 1;
     else if (r1 == rp) w = -1;
     else w = (r0 > r1) - (r0 < r1);
     return w > 0 ? h.con1 : (w < 0 ? -h.con0 : 0);
 }
 
-__device__ __forceinline__ void leduc_apply(LeducHand& h, int a) {
+__host__ __device__ constexpr __forceinline__ void leduc_apply(LeducHand& h, int a) {
     const int me = h.actor, op = 1 - me;
     if (a == 0) {
         h.done = 1;

@@ -370,6 +370,8 @@ int ctx_scratch(void* ctx, int64_t bytes, void** out) {
     return MALIB_OK;
 }
 
+int ctx_policy_seat(const void* ctx, int32_t id) { return static_cast<const malib_ctx*>(ctx)->pols[id].seat; }
+
 void ctx_count_launches(void* ctx, int n) {
     if (ctx) static_cast<malib_ctx*>(ctx)->launches += n;
 }
