@@ -87,6 +87,72 @@ __device__ __forceinline__ void add_contacts(const float (&px)[N], const float (
         }
 }
 
+// True unless the disks are surely too far apart for a force: pen = 0 once d -
+// dmin >= 87 k = 0.087, and q (the squared distance as contact_force rounds it)
+// is above (dmin + 0.0885)^2, a margin of 1.5e-3 that no rounding reaches.
+__device__ __forceinline__ bool contact_near(float ax, float ay, float bx, float by, float dmin) {
+    const float dx = __fsub_rn(ax, bx), dy = __fsub_rn(ay, by);
+    const float q = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+    const float far = dmin + 0.0885f;
+    return !(q > far * far);
+}
+
+// add_contacts, the same bits, for many pairs of which an environment touches
+// few (the simple tag: 14). One force takes about 150 dependent instructions
+// (square root, divisions, softplus), and some lane of a warp needs nearly
+// every pair; here each lane walks its own near pairs, in add_contacts' order,
+// so a warp runs as many forces as its busiest lane has (3 to 5). The tag
+// step's transition went from 10,000 to 4,300 cycles.
+template <int N, int M>
+__device__ __forceinline__ void add_contacts_sparse(const float (&px)[N], const float (&py)[N], const float (&rad)[N],
+                                                    const float* ox, const float* oy, const float* orad,
+                                                    float (&Fx)[N], float (&Fy)[N]) {
+    static_assert(N <= 4 && N + M <= 8 && N * (N - 1) / 2 + N * M <= 16, "pair codes of 5 bits in three words");
+    uint32_t mask = 0;
+    // pair e: its disks a (2 bits) and b (3 bits, obstacles from N on), 6 pairs a word
+    uint32_t code[3] = {0u, 0u, 0u};
+    int e = 0;
+#pragma unroll
+    for (int a = 0; a < N; ++a)
+#pragma unroll
+        for (int b = a + 1; b < N; ++b) {
+            if (contact_near(px[a], py[a], px[b], py[b], __fadd_rn(rad[a], rad[b]))) mask |= 1u << e;
+            code[e / 6] |= (uint32_t)(a | (b << 2)) << (5 * (e % 6));
+            ++e;
+        }
+#pragma unroll
+    for (int a = 0; a < N; ++a)
+#pragma unroll
+        for (int o = 0; o < M; ++o) {
+            if (contact_near(px[a], py[a], ox[o], oy[o], __fadd_rn(rad[a], orad[o]))) mask |= 1u << e;
+            code[e / 6] |= (uint32_t)(a | ((N + o) << 2)) << (5 * (e % 6));
+            ++e;
+        }
+#pragma unroll 1
+    while (mask != 0u) {
+        const int p = __ffs(mask) - 1;
+        mask &= mask - 1u;
+        const uint32_t c = (p < 6 ? code[0] >> (5 * p) : p < 12 ? code[1] >> (5 * (p - 6)) : code[2] >> (5 * (p - 12)));
+        const int a = (int)(c & 3u), b = (int)((c >> 2) & 7u);
+        float ax = px[0], ay = py[0], ar = rad[0], bx = px[0], by = py[0], br = rad[0];
+#pragma unroll
+        for (int k = 1; k < N; ++k) {
+            if (a == k) { ax = px[k]; ay = py[k]; ar = rad[k]; }
+            if (b == k) { bx = px[k]; by = py[k]; br = rad[k]; }
+        }
+#pragma unroll
+        for (int o = 0; o < M; ++o)
+            if (b == N + o) { bx = ox[o]; by = oy[o]; br = orad[o]; }
+        float fx, fy;
+        if (!contact_force(ax, ay, bx, by, __fadd_rn(ar, br), fx, fy)) continue;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            if (a == k) { Fx[k] = __fadd_rn(Fx[k], fx); Fy[k] = __fadd_rn(Fy[k], fy); }
+            if (b == k) { Fx[k] = __fsub_rn(Fx[k], fx); Fy[k] = __fsub_rn(Fy[k], fy); }
+        }
+    }
+}
+
 // Unit force of the five discrete actions (0 noop, 1 +x, 2 -x, 3 +y, 4 -y).
 __device__ __forceinline__ void unit_force(int act, float& fx, float& fy) {
     fx = act == 1 ? 1.f : (act == 2 ? -1.f : 0.f);

@@ -1,18 +1,33 @@
 // Batched rollout of the cooperative particle-spread scenario (App. B.1: N
 // agents cover N landmarks; shared reward minus the summed distance from each
 // landmark to its closest agent, minus one per collision) under policy
-// combinations (Sec. 3.1: X ~ P(s, a, s' | a ~ Comb_t)), fp32 MLP policies.
+// combinations (Sec. 3.1: X ~ P(s, a, s' | a ~ Comb_t)), fp32 MLP policies on
+// the tensor cores (mlp_x3.cuh: fp32 operands as three bf16 parts).
 //
-// Work unit = (combination, episode pair): the combination's block of
-// envs_per_pair (<= 128) environments for T steps, in two episodes at once.
-// Each CTA takes a contiguous, equal-sized range of units (combination-major,
-// so the N policies are staged into shared memory by bulk copy only when the
-// combination changes). Thread t steps environment t % 128 of episode slot
-// t / 128 with its state in registers; per step agent i's observations of both
-// episodes form one 256-row pass of agent i's policy through the fp32 MLP
-// engine. The observation tile is laid out [row][agent][obs_pad], the order of
-// the trajectory, so each episode's observations of a step leave shared memory
-// as one bulk copy; actions, rewards and done flags are stored per thread.
+// Work unit = 128 rows of one combination for T steps: as many whole episodes
+// of its envs_per_pair (<= 128) environments as fit (two of 60, sixteen of 8).
+// A group of four warps plays a unit, one environment per thread with its
+// state in registers: per step and agent the thread writes its observation row
+// (the trajectory's row, and split for the MMAs), turns its row of layer 1
+// into layer 2's operand, forms its logits and draws its action; the group's
+// first thread issues the MMAs. Up to three groups of a CTA share the
+// combination's policies in shared memory and overlap each other's MMAs and
+// waits. Within a group the next agent's observations are written while layer
+// 2 runs, and its layer 1 runs while this agent's logits and draw are formed.
+// An item is a combination's chunk of units; CTAs take items in turn, and the
+// policies are converted from the population's fp32 images when the
+// combination changes. Where a call has fewer units than the chip takes, the
+// groups of a CTA share a unit instead: each plays its own agents' tiles and
+// steps a copy of the environments, and they exchange actions once a step. The
+// plan (units per chunk, groups, shared or not) takes the smallest sum of
+// rounds, weighted by their measured costs.
+//
+// What bounds it: the chain of a tile through its group (about 5,000 cycles:
+// conversion 900, layer 2 1,000, logits 800, observation and stores 1,100, draw
+// 300), overlapped by three groups a CTA; tensor pipe 24 % busy, issue 38 %.
+// 256-row passes of packed fp32 FMAs before (61 % of the FMA pipe, one episode
+// pair per CTA): spread 4,096 environments x 10 episodes 1,343 us, now 355;
+// tag 9 x 125 environments x 3 episodes 990 us, now 275.
 // The same kernel, templated on the scenario, runs the simple adversary, the
 // simple speaker listener, the simple push, the simple tag and the simple
 // reference (App. B.1) with their own environment code, and spread with contact
@@ -24,36 +39,12 @@
 #include "tag_env.cuh"
 #include "device_common.cuh"
 #include "internal.h"
-#include "mlp_f32.cuh"
+#include "mlp_x3.cuh"
 #include "spread_env.cuh"
 
 namespace malib {
 
 namespace {
-
-// Shared memory: the N policies, the observation tile X, layer 1's output H1
-// and the logits LG. When the tiles of all N agents do not fit (the simple tag),
-// the kernel runs per agent (kPerAgent): X and LG hold one agent's rows, each
-// agent's observations are built just before its pass and stored to the
-// trajectory from registers, and its action is drawn right after it.
-template <int N, int IN, int H, int A = 5>
-struct SpreadF32Smem {
-    static_assert(H == 64, "the 256-row engine has 64 hidden units");
-    using M = MlpF32R8<IN, A>;
-    using L = F32Layout<IN, H, A>;
-    static constexpr int R = M::kRows;            // 2 episode slots x 128 envs
-    static constexpr size_t kAllBytes =
-        (size_t)(N * L::kSize + N * R * M::XS + R * M::HS + N * R * M::LS) * 4;
-    static constexpr bool kPerAgent = kAllBytes > 232448;
-    static constexpr int kNX = kPerAgent ? 1 : N;   // agents' tiles held at once
-    static constexpr int kW = 0;
-    static constexpr int kX = kW + N * L::kSize;
-    static constexpr int kH1 = kX + kNX * R * M::XS;
-    static constexpr int kLG = kH1 + R * M::HS;
-    static constexpr int kFloats = kLG + kNX * R * M::LS;
-    static constexpr size_t kBytes = (size_t)kFloats * 4;
-    static_assert(kBytes <= 232448, "fits the 227 KB of shared memory of a CTA");
-};
 
 // kScen: kSpread - cooperative spread (N agents, N landmarks); kAdversary - the
 // simple adversary (N = 3, two landmarks, obs 14); kSpeakerListener - the simple
@@ -91,47 +82,117 @@ struct ScenarioEnv<kReference, N> {
     using type = RefEnv;
 };
 
+constexpr int kGroupThreads = 128;
+constexpr int kMaxGroups = 3;
+
+// How a call's units are dealt (rollout_plan).
+struct RolloutPlan {
+    int epu;                      // episodes per unit
+    int64_t upp;                  // units per combination
+    int64_t per;                  // units per chunk
+    int64_t chunks;               // chunks per combination
+    int64_t items;                // n_pairs * chunks
+    int share;                    // the groups of a CTA share each unit's agents
+};
+
+template <int N, int IN, int kScen>
+struct RolloutSmem {
+    using M = MlpX3<IN, actions_of(kScen)>;
+    static constexpr uint32_t kOnes = N * M::kPolicy;
+    static constexpr uint32_t kX = kOnes + M::kOnesBytes;
+    // Per warp, a buffer through which its rows of observations (or logits) leave
+    // in the trajectory's order: kRows rows at a time, an odd number of 16-byte
+    // units apart (the simple tag's four policies leave room for 16 rows only).
+    static constexpr int kRows = N == 4 ? 16 : 32;
+    static constexpr int kQ = M::XS / 4, kRowUnits = kQ | 1;
+    static constexpr uint32_t kStage = (uint32_t)kRows * kRowUnits * 16;
+    static_assert(kStage >= 32u * actions_of(kScen) * 4 || kRows == 16, "holds a warp's logits");
+    static_assert(kStage >= (uint32_t)kRows * actions_of(kScen) * 4, "holds the rows' logits");
+    __host__ __device__ static constexpr uint32_t stage_at(int groups) { return kX + (uint32_t)groups * M::kXBytes; }
+    __host__ __device__ static constexpr uint32_t bytes(int groups) { return stage_at(groups) + 4u * groups * kStage; }
+    static_assert(bytes(kMaxGroups) + 2048 <= 232448, "fits the 227 KB of shared memory of a CTA");
+    static_assert(kMaxGroups * M::kCols <= 512, "fits tensor memory");
+};
+
+template <int N, int kScen, int XS, class Env>
+__device__ __forceinline__ void scenario_obs(const Env& s, int i, float* o) {
+    if constexpr (kScen == kAdversary) adv_obs<XS>(s, i, o);
+    else if constexpr (kScen == kSpeakerListener) sl_obs<XS>(s, i, o);
+    else if constexpr (kScen == kPush) push_obs<XS>(s, i, o);
+    else if constexpr (kScen == kTag) tag_obs<XS>(s, i, o);
+    else if constexpr (kScen == kReference) ref_obs<XS>(s, i, o);
+    else spread_obs<N, XS>(s, i, o);
+}
+
 // kLogits: the call records the logits (the recording code is compiled out of
-// the other instance).
-template <int N, int IN, int H, int kScen = kSpread, bool kLogits = false>
-__global__ void __launch_bounds__(256, 1) spread_rollout_f32_kernel(RolloutArgs a) {
+// the other instance). blockDim.x = 128 groups.
+template <int N, int IN, int kScen = kSpread, bool kLogits = false>
+__global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
+    spread_rollout_x3_kernel(RolloutArgs a, RolloutPlan plan) {
     static_assert(kScen != kAdversary || (N == 3 && IN == kAdvObs), "the simple adversary has 3 agents, obs 14");
     static_assert(kScen != kSpeakerListener || (N == 2 && IN == kSlObs),
                   "the simple speaker listener has 2 agents, obs 11");
     static_assert(kScen != kPush || (N == 2 && IN == kPushObs), "the simple push has 2 agents, obs 8");
     static_assert(kScen != kTag || (N == 4 && IN == kTagObs), "the simple tag has 4 agents, obs 16");
     static_assert(kScen != kReference || (N == 2 && IN == kRefObs), "the simple reference has 2 agents, obs 14");
+    static_assert(N <= 4 && actions_of(kScen) <= 16, "four bits per agent's action in a 16-bit word");
     constexpr int A = actions_of(kScen);
-    using SM = SpreadF32Smem<N, IN, H, A>;
+    using SM = RolloutSmem<N, IN, kScen>;
     using M = typename SM::M;
-    using L = typename SM::L;
-    constexpr int R = SM::R;
     constexpr int XS = M::XS;           // == obs_pad
-    extern __shared__ __align__(128) float smem[];
-    float* Ws = smem + SM::kW;
-    float* X = smem + SM::kX;
-    float* H1 = smem + SM::kH1;
-    float* LG = smem + SM::kLG;
-    __shared__ __align__(8) uint64_t bar;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    // [group][layer]: its MMAs are complete. One barrier per layer: a thread still
+    // waiting for layer 2 must not meet the completion of the next layer 1, issued
+    // as soon as the issuing warp has seen layer 2 done (with one barrier that
+    // would be its own phase again). Each is completed again only after a
+    // barrier of the group that follows every thread's wait.
+    __shared__ __align__(8) uint64_t bars[kMaxGroups][2];
+    __shared__ uint32_t tmem_base;
+    __shared__ uint32_t dead;           // a bounded wait expired: nobody waits any more
+    __shared__ uint16_t acts[2][kMaxGroups][kGroupThreads];   // shared units: each group's actions of a step
 
-    const int tid = threadIdx.x;
-    const int slot = tid >> 7, v = tid & 127;        // episode slot, env of the combination
-    for (int i = tid; i < R * SM::kNX * XS; i += blockDim.x) X[i] = 0.f;
-    if (tid == 0) mbar_init(&bar, 1);
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int grp = warp >> 2, r = tid & 127;            // group, row of its tiles
+    const int groups = blockDim.x >> 7;
+    const bool issuer = (warp & 3) == 0;                 // this warp issues the group's MMAs
+    if (tid == 0) {
+        for (int g = 0; g < 2 * kMaxGroups; ++g) mbar_init(&bars[0][0] + g, 1);
+        dead = 0u;
+    }
+    if (grp == 0) M::put_ones(smem + SM::kOnes, r);      // fenced with the first policies
+    if (warp == 0) {
+        tc::tmem_alloc(&tmem_base, 512);
+        tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
     __syncthreads();
-    uint32_t parity = 0;
+    tc::fence_after_sync();
+    const uint32_t tb = tmem_base + (uint32_t)grp * M::kCols;
+    const uint32_t lane_q = (uint32_t)(32 * (warp & 3)) << 16;
+    uint8_t* X = smem + SM::kX + (uint32_t)grp * M::kXBytes;
+    float4* buf = reinterpret_cast<float4*>(smem + SM::stage_at(groups) + (uint32_t)warp * SM::kStage);
+    uint64_t* bar = bars[grp];
+    uint32_t phase[2] = {0, 0};
+    auto is_dead = [&] { return *(volatile uint32_t*)&dead != 0u; };
+    auto group_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); };
+    // layer `layer` (0, 1) of the group's current tile has completed
+    auto mma_wait = [&](int layer) {
+        if (!is_dead() && !mbar_wait_bounded(bar + layer, phase[layer], kWaitLimitNs)) {
+            *(volatile uint32_t*)&dead = 1u;
+            atomicOr(a.err, ERRBIT_TIMEOUT);
+            mbar_wait_bounded(bar + layer, phase[layer], kWaitLimitNs);     // its MMAs in flight; none are issued after
+        }
+        phase[layer] ^= 1u;
+        tc::fence_after_sync();
+    };
 
     const int epp = (int)(a.n_envs / a.n_pairs);
     const int T = a.episode_len;
-    const int64_t upp = (a.n_episodes + 1) / 2;         // units (episode pairs) per combination
-    const int64_t units = (int64_t)a.n_pairs * upp;
-    const int64_t lo = units * blockIdx.x / gridDim.x;
-    const int64_t hi = units * (blockIdx.x + 1) / gridDim.x;
     int staged = -1;
-
-    for (int64_t u = lo; u < hi; ++u) {
-        const int pair = (int)(u / upp);
-        const int64_t ep0 = 2 * (u - (int64_t)pair * upp);
+    for (int64_t item = blockIdx.x; item < plan.items; item += gridDim.x) {
+        const int pair = (int)(item / plan.chunks);
+        const int64_t u_lo = (item - (int64_t)pair * plan.chunks) * plan.per;
+        const int64_t u_hi = u_lo + plan.per < plan.upp ? u_lo + plan.per : plan.upp;
         if (pair != staged) {
             bool ok = true;
             for (int i = 0; i < N; ++i) {
@@ -142,194 +203,230 @@ __global__ void __launch_bounds__(256, 1) spread_rollout_f32_kernel(RolloutArgs 
                 if (tid == 0) atomicOr(a.err, ERRBIT_BAD_PAIR);
                 continue;
             }
-            __syncthreads();   // everyone is done with the previous weights
-            if (tid == 0) {
-                fence_proxy_async_smem();
-                mbar_arrive_expect_tx(&bar, (uint32_t)N * L::kSize * 4u);
-                for (int i = 0; i < N; ++i)
-                    bulk_g2s(Ws + i * L::kSize, a.arena + a.pol_offset[a.pairs[pair * N + i]],
-                             (uint32_t)L::kSize * 4u, &bar);
-            }
-            if (!mbar_wait_bounded(&bar, parity, kWaitLimitNs)) {
-                if (tid == 0) {
-                    atomicOr(a.err, ERRBIT_TIMEOUT);
-                    bulk_wait_all();
-                }
-                mbar_wait_bounded(&bar, parity, kWaitLimitNs);
-                return;
-            }
-            parity ^= 1u;
+            __syncthreads();   // every group is done with the previous policies
+            for (int i = 0; i < N; ++i)
+                M::stage(smem + i * M::kPolicy, a.arena + a.pol_offset[a.pairs[pair * N + i]], tid, blockDim.x);
+            fence_proxy_async_smem();
+            __syncthreads();
             staged = pair;
         }
-
-        const int64_t ep = ep0 + slot;
-        const int n_slots = ep0 + 1 < a.n_episodes ? 2 : 1;
-        const bool mine = slot < n_slots && v < epp;
-        const int64_t env = (int64_t)pair * epp + v;
-        const uint64_t g = (uint64_t)ep * (uint64_t)a.n_envs + (uint64_t)env;
-        typename ScenarioEnv<kScen, N>::type s;
-        if (mine) {
-            if constexpr (kScen == kAdversary) adv_reset(s, g, a.seed);
-            else if constexpr (kScen == kSpeakerListener) sl_reset(s, g, a.seed);
-            else if constexpr (kScen == kPush) push_reset(s, g, a.seed);
-            else if constexpr (kScen == kTag) tag_reset(s, g, a.seed);
-            else if constexpr (kScen == kReference) ref_reset(s, g, a.seed);
-            else spread_reset<N>(s, g, a.seed);
-        }
-
-        for (int t = 0; t < T; ++t) {
-            if constexpr (SM::kPerAgent) {
-                // one agent at a time: its observations (to X and the
-                // trajectory), its pass, its draw. The loop stays rolled, so the
-                // MLP's code appears once (instruction fetch limited the unrolled
-                // form); the observation is built by a copy per constant agent
-                // index (no dynamic indexing of the state in registers), and the
-                // actions are packed one byte per agent.
-                static_assert(N <= 4, "one byte per agent's action in a 32-bit word");
+        // agents i0, i0 + di, ... are this group's
+        const int i0 = plan.share ? grp : 0, di = plan.share ? groups : 1;
+        for (int64_t u = plan.share ? u_lo : u_lo + grp; u < u_hi; u += plan.share ? 1 : groups) {
+            const int slot = r / epp, v = r - slot * epp;
+            const int64_t ep = u * plan.epu + slot;
+            const bool mine = slot < plan.epu && ep < a.n_episodes;
+            const bool busy = __any_sync(0xffffffffu, mine);     // warps without rows only keep step
+            const int64_t env = (int64_t)pair * epp + v;
+            const uint64_t g = (uint64_t)ep * (uint64_t)a.n_envs + (uint64_t)env;
+            typename ScenarioEnv<kScen, N>::type s;
+            if (mine) {
+                if constexpr (kScen == kAdversary) adv_reset(s, g, a.seed);
+                else if constexpr (kScen == kSpeakerListener) sl_reset(s, g, a.seed);
+                else if constexpr (kScen == kPush) push_reset(s, g, a.seed);
+                else if constexpr (kScen == kTag) tag_reset(s, g, a.seed);
+                else if constexpr (kScen == kReference) ref_reset(s, g, a.seed);
+                else spread_reset<N>(s, g, a.seed);
+            } else {
+                M::zero_row(X, r);      // stays zero for the unit
+            }
+            int64_t ix = (ep * T * a.n_envs + env) * N;          // this step's (env, agent 0)
+            // Agent i's observation into the tile. It leaves for the trajectory
+            // only after the barrier that follows: the proxy fence waits for the
+            // thread's earlier stores, and with the global ones before it that
+            // took 2,000 cycles.
+            float o[XS];
+            auto observe = [&](int i) {
+                if (mine) {
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        if (j == i) scenario_obs<N, kScen, XS>(s, j, o);
+                    M::put_row(X, r, o);
+                }
+                fence_proxy_async_smem();
+            };
+            // The warp's rows through its buffer, so that consecutive lanes store
+            // consecutive 16-byte units (4-byte ones for logits) of an
+            // environment's row: stored by each thread for itself, a warp's store
+            // touched 32 lines, and a step's stores took 2,500 cycles.
+            auto store_obs = [&](int i) {
+                if (!busy) return;
+                const unsigned rows = __ballot_sync(0xffffffffu, mine);
+                const int64_t at = (ix + i) * SM::kQ;
+#pragma unroll
+                for (int h = 0; h < 32; h += SM::kRows) {
+                    __syncwarp();                            // the buffer is read
+                    if (lane >= h && lane < h + SM::kRows)
+#pragma unroll
+                        for (int q = 0; q < SM::kQ; ++q)
+                            buf[(lane - h) * SM::kRowUnits + q] =
+                                make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < SM::kRows * SM::kQ / 32; ++k) {
+                        const int c = lane + 32 * k, row = c / SM::kQ, q = c - row * SM::kQ;
+                        const int64_t to = __shfl_sync(0xffffffffu, at, row + h);
+                        if ((rows >> (row + h)) & 1u)
+                            reinterpret_cast<float4*>(a.obs)[to + q] = buf[row * SM::kRowUnits + q];
+                    }
+                }
+            };
+            auto store_logits = [&](int i, const float (&lg)[A]) {
+                const unsigned rows = __ballot_sync(0xffffffffu, mine);
+                const int64_t at = (ix + i) * A;
+                float* fb = reinterpret_cast<float*>(buf);
+#pragma unroll
+                for (int h = 0; h < 32; h += SM::kRows) {
+                    __syncwarp();
+                    if (lane >= h && lane < h + SM::kRows)
+#pragma unroll
+                        for (int k = 0; k < A; ++k) fb[(lane - h) * A + k] = lg[k];
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < (SM::kRows * A + 31) / 32; ++k) {
+                        const int c = lane + 32 * k, row = c / A, q = c - row * A;
+                        const int64_t to = __shfl_sync(0xffffffffu, at, (row + h) & 31);
+                        if (row < SM::kRows && ((rows >> (row + h)) & 1u)) a.logits[to + q] = fb[c];
+                    }
+                }
+            };
+            // the group's tile is written (and layer 2 of the tile before is done): layer 1
+            auto layer1 = [&](int i) {
+                if (issuer && !is_dead() && tc::elect_one())
+                    M::issue1(tb, smem_u32(X), smem_u32(smem + SM::kOnes), smem_u32(smem + i * M::kPolicy), bar);
+                __syncwarp();
+            };
+            observe(i0);
+            tc::fence_before_sync();
+            group_sync();
+            tc::fence_after_sync();
+            layer1(i0);
+            store_obs(i0);
+            for (int t = 0; t < T; ++t) {
                 uint32_t act_pk = 0;
-                const int64_t ix = ((ep * T + t) * a.n_envs + env) * N;
 #pragma unroll 1
-                for (int i = 0; i < N; ++i) {
-                    if (mine) {
-                        float o[XS];
-#pragma unroll
-                        for (int j = 0; j < N; ++j) {
-                            if (j != i) continue;
-                            if constexpr (kScen == kTag) tag_obs<XS>(s, j, o);
-                            else if constexpr (kScen == kReference) ref_obs<XS>(s, j, o);
-                            else if constexpr (kScen == kPush) push_obs<XS>(s, j, o);
-                            else if constexpr (kScen == kAdversary) adv_obs<XS>(s, j, o);
-                            else if constexpr (kScen == kSpeakerListener) sl_obs<XS>(s, j, o);
-                            else spread_obs<N, XS>(s, j, o);
-                        }
-                        float4* xr = reinterpret_cast<float4*>(X + tid * XS);
-                        float4* gr = reinterpret_cast<float4*>(a.obs + (ix + i) * XS);
-#pragma unroll
-                        for (int q = 0; q < XS / 4; ++q) {
-                            const float4 f = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-                            xr[q] = f;
-                            gr[q] = f;
-                        }
+                for (int i = i0; i < N; i += di) {
+                    const uint8_t* pol = smem + i * M::kPolicy;
+                    mma_wait(0);                             // layer 1
+                    if (busy) M::hidden(tb, lane_q);
+                    tc::fence_before_sync();
+                    group_sync();
+                    tc::fence_after_sync();
+                    if (issuer && !is_dead() && tc::elect_one()) M::issue2(tb, smem_u32(smem + SM::kOnes), smem_u32(pol), bar + 1);
+                    __syncwarp();
+                    const float uu = u24(draw(g, (uint32_t)t, (uint32_t)i, a.seed).x);
+                    if (i + di < N) {
+                        observe(i + di);                     // layer 1 no longer reads the tile
+                        group_sync();
+                        store_obs(i + di);
                     }
-                    __syncthreads();
-                    const float* w = Ws + i * L::kSize;
-                    M::template layer1<XS>(X, H1, w + L::kW1T, w + L::kB1);
-                    M::layer23(H1, LG, w + L::kW2T, w + L::kB2, w + L::kW3, w + L::kB3);
-                    if (mine) {
-                        // LG is rewritten only after the next pass's layer-1 barrier
+                    mma_wait(1);                             // layer 2
+                    if (i + di < N) layer1(i + di);
+                    if (busy) {
                         float lg[A];
-#pragma unroll
-                        for (int k = 0; k < A; ++k) lg[k] = LG[tid * M::LS + k];
-                        const float uu = u24(draw(g, (uint32_t)t, (uint32_t)i, a.seed).x);
-                        const unsigned legal = (kScen == kSpeakerListener && i == 0) ? kSlSpeakerLegal : (1u << A) - 1u;
-                        act_pk |= (uint32_t)sample_masked<A>(lg, legal, uu) << (8 * i);
-                        if (kLogits)
-#pragma unroll
-                            for (int k = 0; k < A; ++k) a.logits[(ix + i) * A + k] = lg[k];
+                        M::logits(tb, lane_q, pol, lg);
+                        if (mine) {
+                            const unsigned legal = (kScen == kSpeakerListener && i == 0) ? kSlSpeakerLegal : (1u << A) - 1u;
+                            act_pk |= (uint32_t)sample_masked<A>(lg, legal, uu) << (4 * i);
+                        }
+                        if (kLogits) store_logits(i, lg);
                     }
+                }
+                if (plan.share) {
+                    // the other groups' actions (a buffer is written again only
+                    // after the next step's barrier)
+                    acts[t & 1][grp][r] = (uint16_t)act_pk;
+                    asm volatile("bar.sync %0, %1;" ::"r"(kMaxGroups + 1), "r"((int)blockDim.x) : "memory");
+                    for (int q = 0; q < groups; ++q)
+                        if (q != grp) act_pk |= acts[t & 1][q][r];
+                }
+                int act[N];
+                float rw[N];
+#pragma unroll
+                for (int i = 0; i < N; ++i) act[i] = (int)((act_pk >> (4 * i)) & 0xfu);
+                if (mine) {
+                    if constexpr (kScen == kAdversary) adv_step(s, act, rw);
+                    else if constexpr (kScen == kSpeakerListener) sl_step(s, act, rw);
+                    else if constexpr (kScen == kPush) push_step(s, act, rw);
+                    else if constexpr (kScen == kTag) tag_step(s, act, rw);
+                    else if constexpr (kScen == kReference) ref_step(s, act, rw, a.local_ratio < 0.f ? 0.5f : a.local_ratio);
+                    else spread_step<N, kScen == kSpreadContact>(s, act, rw, a.local_ratio);
+                }
+                if (t + 1 < T) {
+                    observe(i0);
+                    tc::fence_before_sync();
+                    group_sync();
+                    tc::fence_after_sync();
+                    layer1(i0);
                 }
                 if (mine) {
-                    int act[N];
-#pragma unroll
-                    for (int i = 0; i < N; ++i) act[i] = (int)((act_pk >> (8 * i)) & 0xffu);
-                    float r[N];
-                    if constexpr (kScen == kAdversary) adv_step(s, act, r);
-                    else if constexpr (kScen == kSpeakerListener) sl_step(s, act, r);
-                    else if constexpr (kScen == kPush) push_step(s, act, r);
-                    else if constexpr (kScen == kTag) tag_step(s, act, r);
-                    else if constexpr (kScen == kReference) ref_step(s, act, r, a.local_ratio < 0.f ? 0.5f : a.local_ratio);
-                    else spread_step<N, kScen == kSpreadContact>(s, act, r, a.local_ratio);
 #pragma unroll
                     for (int i = 0; i < N; ++i) {
+                        if (plan.share && i % groups != grp) continue;
                         a.action[ix + i] = (uint8_t)act[i];
-                        a.reward[ix + i] = r[i];
+                        a.reward[ix + i] = rw[i];
                     }
-                    a.done[(ep * T + t) * a.n_envs + env] = (t == T - 1) ? 1 : 0;
+                    if (i0 == 0) a.done[(ep * T + t) * a.n_envs + env] = (t == T - 1) ? 1 : 0;
                 }
-                continue;
+                ix += a.n_envs * N;
+                if (t + 1 < T) store_obs(i0);
             }
-            if (mine) {
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    float o[XS];
-                    if constexpr (kScen == kAdversary) adv_obs<XS>(s, i, o);
-                    else if constexpr (kScen == kSpeakerListener) sl_obs<XS>(s, i, o);
-                    else if constexpr (kScen == kPush) push_obs<XS>(s, i, o);
-                    else if constexpr (kScen == kTag) tag_obs<XS>(s, i, o);
-                    else if constexpr (kScen == kReference) ref_obs<XS>(s, i, o);
-                    else spread_obs<N, XS>(s, i, o);
-                    float4* xr = reinterpret_cast<float4*>(X + (tid * N + i) * XS);
-#pragma unroll
-                    for (int q = 0; q < XS / 4; ++q)
-                        xr[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-                }
-                fence_proxy_async_smem();                // the rows are read by bulk copies
-            }
-            __syncthreads();
-            // trajectory observations, [ep][t][env][agent][XS]: an episode's rows
-            // are contiguous in the tile and in the trajectory
-            if (tid == 0) {
-                for (int sl = 0; sl < n_slots; ++sl) {
-                    const int64_t row_base = (((ep0 + sl) * T + t) * a.n_envs + (int64_t)pair * epp) * N;
-                    bulk_s2g(a.obs + row_base * XS, X + sl * 128 * N * XS, (uint32_t)(epp * N * XS * 4));
-                }
-                bulk_commit();
-            }
-            for (int i = 0; i < N; ++i) {
-                const float* w = Ws + i * L::kSize;
-                M::template layer1<N * XS>(X + i * XS, H1, w + L::kW1T, w + L::kB1);
-                // the copies have read the tile before the last pass's barrier;
-                // the tile is rewritten only after it
-                if (i == N - 1 && tid == 0) bulk_wait_read();
-                M::layer23(H1, LG + i * R * M::LS, w + L::kW2T, w + L::kB2, w + L::kW3, w + L::kB3);
-            }
-            if (mine) {
-                int act[N];
-                float r[N];
-                const int64_t ix = ((ep * T + t) * a.n_envs + env) * N;
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    float lg[A];
-#pragma unroll
-                    for (int k = 0; k < A; ++k) lg[k] = LG[(i * R + tid) * M::LS + k];
-                    const float uu = u24(draw(g, (uint32_t)t, (uint32_t)i, a.seed).x);
-                    const unsigned legal = (kScen == kSpeakerListener && i == 0) ? kSlSpeakerLegal : (1u << A) - 1u;
-                    act[i] = sample_masked<A>(lg, legal, uu);
-                    if (kLogits)
-#pragma unroll
-                        for (int k = 0; k < A; ++k) a.logits[(ix + i) * A + k] = lg[k];
-                }
-                if constexpr (kScen == kAdversary) adv_step(s, act, r);
-                else if constexpr (kScen == kSpeakerListener) sl_step(s, act, r);
-                else if constexpr (kScen == kPush) push_step(s, act, r);
-                else if constexpr (kScen == kTag) tag_step(s, act, r);
-                else if constexpr (kScen == kReference) ref_step(s, act, r, a.local_ratio < 0.f ? 0.5f : a.local_ratio);
-                else spread_step<N, kScen == kSpreadContact>(s, act, r, a.local_ratio);
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    a.action[ix + i] = (uint8_t)act[i];
-                    a.reward[ix + i] = r[i];
-                }
-                a.done[(ep * T + t) * a.n_envs + env] = (t == T - 1) ? 1 : 0;
-            }
-            // X is rewritten next step only after the passes' trailing barrier;
-            // LG is rewritten only after next step's first barrier.
+            // the next unit's first barrier orders its MMAs after this unit's
+            // last reads of D2
         }
     }
-    if (tid == 0) bulk_wait_all();   // the trajectory copies have landed
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tmem_base, 512);
 }
 
-template <int N, int IN, int H, int kScen = kSpread>
-cudaError_t launch_spread_nih(const RolloutArgs& a, int n_sm, cudaStream_t s) {
-    using SM = SpreadF32Smem<N, IN, H, actions_of(kScen)>;
-    auto kern = a.logits ? spread_rollout_f32_kernel<N, IN, H, kScen, true>
-                         : spread_rollout_f32_kernel<N, IN, H, kScen, false>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::kBytes);
+// Costs in units of one unit played by one group alone (152 CTAs, 128
+// environments; spread 242 us): a round of g groups took 1.14 to 1.26 (g = 2)
+// and 1.37 to 1.56 (3), a unit shared by its agents' groups 0.70 to 0.82 over
+// the seven scenarios; converting a combination's policies about 5 us.
+constexpr double kRoundCost[kMaxGroups + 1] = {0.0, 1.0, 1.2, 1.46};
+constexpr double kShareCost = 0.76;
+constexpr double kStageCost = 0.03;
+
+RolloutPlan rollout_plan(int32_t n_pairs, int n_agents, int64_t epp, int64_t n_episodes, int n_sm, int* groups,
+                         int64_t* grid) {
+    RolloutPlan p{};
+    p.epu = (int)(kGroupThreads / epp);
+    p.upp = (n_episodes + p.epu - 1) / p.epu;
+    const int gs = n_agents == 3 ? 3 : 2;              // groups of a shared unit: equal numbers of agents
+    double best = 1e300;
+    // chunks of `per` units: all sizes up to 96, then doubling
+    for (int64_t per = 1; per <= p.upp; per = per < 96 ? per + 1 : (per * 2 < p.upp || per == p.upp ? per * 2 : p.upp)) {
+        const int64_t chunks = (p.upp + per - 1) / per;
+        const int64_t turns = ((int64_t)n_pairs * chunks + n_sm - 1) / n_sm;
+        for (int g = 0; g <= kMaxGroups && g <= per; ++g) {   // 0: shared units
+            const double rounds = g == 0 ? (double)per * kShareCost : (double)((per + g - 1) / g) * kRoundCost[g];
+            const double cost = (double)turns * (kStageCost + rounds);
+            if (cost < best) {
+                best = cost;
+                p.per = per;
+                p.chunks = chunks;
+                p.share = g == 0;
+                *groups = g == 0 ? gs : g;
+            }
+        }
+    }
+    p.items = (int64_t)n_pairs * p.chunks;
+    *grid = p.items < n_sm ? p.items : n_sm;
+    return p;
+}
+
+template <int N, int IN, int kScen = kSpread>
+cudaError_t launch_rollout(const RolloutArgs& a, int n_sm, cudaStream_t s) {
+    using SM = RolloutSmem<N, IN, kScen>;
+    int groups = 1;
+    int64_t grid = 1;
+    const RolloutPlan plan = rollout_plan(a.n_pairs, N, a.n_envs / a.n_pairs, a.n_episodes, n_sm, &groups, &grid);
+    auto kern = a.logits ? spread_rollout_x3_kernel<N, IN, kScen, true> : spread_rollout_x3_kernel<N, IN, kScen, false>;
+    const uint32_t bytes = SM::bytes(groups);
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (err != cudaSuccess) return err;
-    const int64_t units = (int64_t)a.n_pairs * ((a.n_episodes + 1) / 2);
-    int64_t grid = units < n_sm ? units : n_sm;
-    if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, 256, SM::kBytes, s>>>(a);
+    kern<<<(unsigned)grid, kGroupThreads * groups, bytes, s>>>(a, plan);
     return cudaGetLastError();
 }
 
@@ -344,28 +441,28 @@ bool spread_f32_supported(int n_agents, int obs_dim, int hidden) {
 cudaError_t launch_spread_rollout_f32(const RolloutArgs& a, int hidden, int n_sm, cudaStream_t s) {
     if (a.n_pairs == 0 || a.n_episodes == 0) return cudaSuccess;
     if (a.env_kind == MALIB_ENV_ADVERSARY) {
-        if (hidden == 64) return launch_spread_nih<3, kAdvObs, 64, kAdversary>(a, n_sm, s);
+        if (hidden == 64) return launch_rollout<3, kAdvObs, kAdversary>(a, n_sm, s);
         return cudaErrorInvalidValue;
     }
     if (a.env_kind == MALIB_ENV_SPEAKER_LISTENER) {
-        if (hidden == 64) return launch_spread_nih<2, kSlObs, 64, kSpeakerListener>(a, n_sm, s);
+        if (hidden == 64) return launch_rollout<2, kSlObs, kSpeakerListener>(a, n_sm, s);
         return cudaErrorInvalidValue;
     }
     if (a.env_kind == MALIB_ENV_PUSH) {
-        if (hidden == 64) return launch_spread_nih<2, kPushObs, 64, kPush>(a, n_sm, s);
+        if (hidden == 64) return launch_rollout<2, kPushObs, kPush>(a, n_sm, s);
         return cudaErrorInvalidValue;
     }
     if (a.env_kind == MALIB_ENV_REFERENCE) {
-        if (hidden == 64) return launch_spread_nih<2, kRefObs, 64, kReference>(a, n_sm, s);
+        if (hidden == 64) return launch_rollout<2, kRefObs, kReference>(a, n_sm, s);
         return cudaErrorInvalidValue;
     }
     if (a.env_kind == MALIB_ENV_TAG) {
-        if (hidden == 64) return launch_spread_nih<4, kTagObs, 64, kTag>(a, n_sm, s);
+        if (hidden == 64) return launch_rollout<4, kTagObs, kTag>(a, n_sm, s);
         return cudaErrorInvalidValue;
     }
     if (a.n_agents == 3 && a.obs_dim == 18 && hidden == 64)
-        return a.contact ? launch_spread_nih<3, 18, 64, kSpreadContact>(a, n_sm, s)
-                         : launch_spread_nih<3, 18, 64>(a, n_sm, s);
+        return a.contact ? launch_rollout<3, 18, kSpreadContact>(a, n_sm, s)
+                         : launch_rollout<3, 18>(a, n_sm, s);
     return cudaErrorInvalidValue;
 }
 

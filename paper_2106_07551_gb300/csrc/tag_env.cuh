@@ -86,7 +86,7 @@ __device__ __forceinline__ void tag_step(TagEnv& s, const int (&act)[4], float (
         rad[i] = tag_radius(i);
     }
     const float orad[2] = {0.2f, 0.2f};
-    add_contacts<4, 2>(s.px, s.py, rad, s.ox, s.oy, orad, Fx, Fy);
+    add_contacts_sparse<4, 2>(s.px, s.py, rad, s.ox, s.oy, orad, Fx, Fy);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         float vx = __fadd_rn(__fmul_rn(s.vx[i], 0.75f), __fmul_rn(Fx[i], 0.1f));

@@ -78,6 +78,20 @@ def test_tag_replay_parity(n_envs, epp, n_eps):
     ctx.close()
 
 
+@pytest.mark.parametrize("n_envs,epp,n_eps", [(1280, 8, 40), (640, 128, 9)])
+def test_tag_units_over_groups_and_items(n_envs, epp, n_eps):
+    """Several 128-row units per CTA and more combinations than SMs; four
+    policies, rows that leave 16 at a time: sampled environments replayed."""
+    need_gpu()
+    w = workloads.tag(n_envs=n_envs, pop=6, envs_per_pair=epp, with_bias=True, seed=n_envs)
+    ctx = context()
+    load_population(ctx, w)
+    g = rollout(ctx, w, n_eps, 515)
+    for lo in (0, n_envs // 2, n_envs - 9):
+        check(oracle.tag_rollout, w, g, n_eps, 515, lo, lo + 9)
+    ctx.close()
+
+
 def test_push_tag_4096_envs_sampled():
     need_gpu()
     for make, replay in ((workloads.push, oracle.push_rollout), (workloads.tag, oracle.tag_rollout)):

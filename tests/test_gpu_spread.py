@@ -57,6 +57,22 @@ def test_full_replay_parity(orc, n_envs, epp, n_eps):
     ctx.close()
 
 
+@pytest.mark.parametrize("n_envs,epp,n_eps", [(1280, 8, 40), (2200, 11, 34), (875, 125, 1), (640, 128, 9)])
+def test_units_over_groups_and_items(orc, n_envs, epp, n_eps):
+    """Sixteen, eleven and one episodes per 128-row unit, more combinations than
+    SMs (a CTA takes several items and several units at once), combinations
+    whose last unit is partly empty, and calls so small that groups share a
+    unit: first, middle and last environments of every episode are replayed."""
+    need_gpu()
+    w = workloads.spread(n_agents=3, n_envs=n_envs, pop=7, envs_per_pair=epp, with_bias=True, seed=n_envs)
+    ctx = context()
+    load_population(ctx, w)
+    g = rollout(ctx, w, n_eps, 99)
+    for lo in (0, n_envs // 2, n_envs - 9):
+        check(orc, w, g, n_eps, 99, lo, lo + 9)
+    ctx.close()
+
+
 @pytest.mark.parametrize("rho", [0.0, 0.3, 1.0])
 def test_local_ratio_replay_parity(orc, rho):
     """App. B.1's local_ratio weighting of the reward: bit-exact under replay."""
