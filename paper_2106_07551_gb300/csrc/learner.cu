@@ -38,7 +38,7 @@
 
 #include "device_common.cuh"
 #include "internal.h"
-#include "mlp_f32.cuh"      // packed fp32 pair helpers (f2_fma: two IEEE fmaf per instruction)
+#include "f32x2.cuh"
 
 namespace malib {
 

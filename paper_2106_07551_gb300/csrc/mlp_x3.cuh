@@ -36,7 +36,7 @@
 #include <cstdint>
 
 #include "device_common.cuh"
-#include "mlp_f32.cuh"
+#include "f32x2.cuh"
 #include "tc_common.cuh"
 
 namespace malib {
@@ -48,18 +48,6 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t& h, uint32_t
     const float r1 = __fsub_rn(v1, __uint_as_float(h & 0xffff0000u));
     m = tc::pack_bf16(r0, r1);
     l = tc::pack_bf16(__fsub_rn(r0, __uint_as_float(m << 16)), __fsub_rn(r1, __uint_as_float(m & 0xffff0000u)));
-}
-
-__device__ __forceinline__ unsigned long long f2_pack(uint32_t lo, uint32_t hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-// Two fp32 additions, each rounded to nearest.
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
 }
 
 template <int IN, int A>

@@ -11,7 +11,7 @@
 // file-scope device array below instead of context-owned memory grown with
 // cudaMallocAsync, and it stages nothing (pair table and output must already
 // be device buffers). The scratch also holds the per-pair hand counters from
-// which the fp32 Leduc kernel's CTAs claim hands.
+// which the fp32 Leduc kernel's CTAs claim work units.
 //
 // The array has room for kNoAllocMaxPairs pairs: (3 * 8192 + 1) x 8 bytes
 // (sums, decision counter, hand counters), 192 KiB + 8 B, held by every GPU

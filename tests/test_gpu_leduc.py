@@ -97,6 +97,42 @@ def test_claimed_hands_across_pairs(orc, n_eps):
     ctx.close()
 
 
+@pytest.mark.parametrize("hidden,n_eps", [(64, 127), (128, 129), (128, 300), (64, 1025)])
+def test_tile_edges(orc, hidden, n_eps):
+    """Hands per unit around the 128-row tile and the two groups' tiles."""
+    need_gpu()
+    w = workloads.leduc(pop=2, hidden=hidden, with_bias=True, seed=n_eps)
+    ctx = context()
+    load_population(ctx, w)
+    pairs = np.tile(w.pair_ids, (40, 1))              # enough pairs that a pair is one unit
+    dump = alloc_eval_dump(MALIB_ENV_LEDUC, len(pairs), n_eps)
+    res = ctx.eval_payoff_ex(pairs, n_eps, 17, MALIB_DUMP_LOGITS, dump=dump, n_dump=n_eps)
+    ctx.sync()
+    w.pair_ids = pairs
+    check_replay(orc, w, res, {k: v.cpu().numpy() for k, v in dump.items()}, n_eps, 17, n_eps, full=True)
+    ctx.close()
+
+
+@pytest.mark.parametrize("action", [1, 2])
+def test_whole_units_that_never_fold(orc, action):
+    """Policies with zero weights that always call, or raise where they may: all
+    8,192 hands of a unit stay alive and act together, and seat 0 acts twice in a
+    row at the second round, so every list fills up."""
+    need_gpu()
+    w = workloads.leduc(pop=1, hidden=64, seed=3)
+    for p in w.policies:
+        p.params[:] = 0.0
+        p.params[-3 + 1] = 50.0
+        p.params[-3 + action] = 100.0
+    ctx = context()
+    load_population(ctx, w)
+    pairs = np.tile(w.pair_ids, (152, 1))
+    res = ctx.eval_payoff(pairs, 8192, 23)
+    ctx.close()
+    ref, _ = orc.leduc_eval([p.params for p in w.policies], w.policies[0].dims, pairs, 8192, 23)
+    np.testing.assert_array_equal(res[:, 2:], ref[:, 2:])
+
+
 def test_full_workload_sampled_replay_and_exact_expectation(orc):
     """8x8 pairs x 65,536 hands in the benchmark's launch configuration."""
     need_gpu()
