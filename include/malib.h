@@ -347,7 +347,7 @@ int malib_meta_fictitious_play(malib_ctx* ctx, const double* payoff, int32_t n_g
 
 /* Exact equilibrium by linear programming (simplex, Bland's rule): value_out
  * [G] = the game value; x_out [G][m], y_out [G][n] one equilibrium (not unique
- * in general). 1 <= m, n <= 512; tableaus larger than 200 KB live in
+ * in general). 1 <= m, n <= 512; tableaus that do not fit on chip live in
  * context-owned device memory. A game that reaches the pivot limit raises
  * MALIB_ENOTCONVERGED at the next malib_sync. */
 int malib_meta_lp_nash(malib_ctx* ctx, const double* payoff, int32_t n_games, int32_t m,

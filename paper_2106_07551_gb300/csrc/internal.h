@@ -240,9 +240,7 @@ cudaError_t launch_fictitious_play(const double* P, int32_t G, int32_t m, int32_
 cudaError_t launch_aggregate(const double* P, int32_t G, int32_t m, int32_t n, int32_t stride,
                              const double* x, const double* y, double* ay, double* xa, double* val,
                              int n_sm, cudaStream_t s);
-int64_t lp_tableau_doubles(int32_t m, int32_t n);
-bool lp_on_chip(int32_t m, int32_t n);
-int lp_grid(int32_t n_games, int n_sm);
+int64_t lp_scratch_bytes(int32_t n_games, int32_t m, int32_t n, int n_sm);   // 0: tableaus fit on chip
 cudaError_t launch_lp_nash(const double* P, int32_t G, int32_t m, int32_t n, int32_t stride,
                            double* x, double* y, double* val, double* scratch, int32_t pivot_limit,
                            int* err, int n_sm, cudaStream_t s);

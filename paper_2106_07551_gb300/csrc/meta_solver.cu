@@ -8,6 +8,7 @@
 // when it fits, cumulative payoffs in registers, and each iteration's argmax /
 // argmin in warp shuffles plus one cross-warp step.
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "malib.h"
@@ -16,9 +17,9 @@ namespace malib {
 
 namespace {
 
-constexpr int kFpThreads = 256;
+constexpr int kFpWarps = 8;                     // warps per side
 constexpr int kFpPer = 4;                       // rows (columns) per thread: m, n <= 1024
-constexpr int kFpMaxDim = kFpThreads * kFpPer;
+constexpr int kFpMaxDim = 32 * kFpWarps * kFpPer;
 constexpr int kSmemLimit = 200 * 1024;          // bytes of payoff / tableau kept on chip
 
 // Order-preserving integer key of a finite double (larger double, larger
@@ -59,25 +60,49 @@ __device__ __forceinline__ Cand warp_pick(Cand a) {
     return a;
 }
 
+// The best candidate of a warp (every lane gets it): the largest key by its high
+// then its low word, then the lowest index, each one warp-wide integer
+// reduction. Five rounds of 64-bit shuffles and selects took about twice as long.
+__device__ __forceinline__ Cand warp_best(Cand a) {
+    const int hi = (int)(a.k >> 32);
+    const unsigned lo = (unsigned)a.k;
+    const int mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const unsigned i = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? (unsigned)a.i : 0xffffffffu);
+    return Cand{((long long)mh << 32) | (long long)ml, (int)i};
+}
+
 // Simultaneous fictitious play: both play policy 0 first; then each plays the
-// first best response to the other's plays so far. u_row[i] = sum over plays
-// of A[i][j_s] and u_col[j] = sum of A[i_s][j] are fp64 sums in play order,
-// held in registers with the play counts (thread t owns rows and columns t,
-// t + blockDim, ...). One CTA barrier per play: every warp publishes its best
-// row and column into a buffer selected by the play's parity, and after the
-// barrier every warp reduces the published candidates itself, so all threads
-// know the next plays. The column player's argmin is the argmax of the
-// negated key.
-template <bool kOnChip>
-__global__ void __launch_bounds__(kFpThreads) fictitious_play_kernel(
+// first best response to the other's plays so far. u_row[i] = sum over plays of
+// A[i][j_s] and u_col[j] = sum of A[i_s][j] are fp64 sums in play order, held in
+// registers. The column player's argmin is the argmax of the negated key.
+//
+// A play is a chain: load, fp64 addition (64 cycles), argmax in the warp (three
+// integer reductions of 24), one CTA barrier, argmax over the side's warps;
+// nothing of the next play can start before. So the two sides are on different
+// warps (two additions would take turns on a scheduler), and after the barrier
+// every thread reads both sides' at most eight candidates from shared memory (a
+// buffer selected by the play's parity, so one barrier per play) and takes the
+// best by a fixed tree; the play counts are compares in registers, off the
+// chain. 64 x 64, one game: 165 ns a play; with both sides on every warp, the
+// argmax by 64-bit shuffles and the candidates reduced again in every warp 575.
+// Warps 0 .. wr - 1 hold the rows (row lane + 32 w + 32 wr k), the rest the
+// columns. K: rows (columns) per thread; W: candidates per side read (1, 2, 4, 8).
+template <bool kOnChip, int K, int W>
+__global__ void __launch_bounds__(64 * W) fictitious_play_kernel(
     const double* __restrict__ P, int32_t n_games, int32_t m, int32_t n, int32_t stride,
-    int64_t T, double* __restrict__ x_out, double* __restrict__ y_out,
+    int64_t T, int32_t wr, double* __restrict__ x_out, double* __restrict__ y_out,
     double* __restrict__ bounds_out) {
     extern __shared__ double sA[];              // [m][ld] when on chip
-    __shared__ Cand red[2][2][8];
+    __shared__ Cand red[2][2][W];               // [play's parity][side][warp]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nt = blockDim.x;
     const int ld = n | 1;                       // odd row stride: column reads hit distinct banks
+    const int side = warp >= wr ? 1 : 0, ws = side ? (nt >> 5) - wr : wr, w = warp - side * wr;
+    const int dim = side ? n : m;
+    // strides of this side's entries and of the other side's policies
+    const int64_t sq = kOnChip ? (side ? 1 : ld) : (int64_t)stride * (side ? 1 : n);
+    const int64_t so = kOnChip ? (side ? ld : 1) : (int64_t)stride * (side ? n : 1);
 
     for (int g = blockIdx.x; g < n_games; g += gridDim.x) {
         const double* Pg = P + (int64_t)g * m * n * stride;
@@ -88,92 +113,117 @@ __global__ void __launch_bounds__(kFpThreads) fictitious_play_kernel(
                 sA[i * ld + j] = Pg[(int64_t)k * stride];
             }
         }
-        if (tid < 32) {
-            const Cand none{kNone, 0x7fffffff};
-            (&red[0][0][0])[tid] = none;
-        }
+        if (tid < 4 * W) (&red[0][0][0])[tid] = Cand{kNone, 0x7fffffff};   // warps that do not exist
         __syncthreads();
-        auto a_at = [&](int i, int j) -> double {
-            return kOnChip ? sA[i * ld + j] : __ldg(Pg + ((int64_t)i * n + j) * stride);
-        };
-        double ur[kFpPer], uc[kFpPer];
-        long long cr[kFpPer], cc[kFpPer];
+        double u[K];
+        long long cnt[K];
+        const double* at[K];
 #pragma unroll
-        for (int k = 0; k < kFpPer; ++k) { ur[k] = 0.0; uc[k] = 0.0; cr[k] = 0; cc[k] = 0; }
-        int it = 0, jt = 0;
-        Cand top{kNone, 0x7fffffff}, bot{kNone, 0x7fffffff};
+        for (int k = 0; k < K; ++k) {
+            const int q = lane + 32 * (w + ws * k);
+            u[k] = 0.0;
+            cnt[k] = 0;
+            at[k] = (kOnChip ? sA : Pg) + (q < dim ? q * sq : 0);
+        }
+        int other = 0, own = 0;
+        Cand best_own{kNone, 0}, best_other{kNone, 0};
         for (int64_t t = 0; t < T; ++t) {
             const int par = (int)(t & 1);
-            Cand br{kNone, 0x7fffffff}, bc{kNone, 0x7fffffff};
+            Cand b{kNone, 0x7fffffff};
 #pragma unroll
-            for (int k = 0; k < kFpPer; ++k) {
-                const int i = tid + k * nt;
-                if (i < m) {
-                    cr[k] += (i == it);
-                    ur[k] += a_at(i, jt);
-                    br = pick(br, Cand{okey(ur[k]), i});
-                }
-                if (i < n) {
-                    cc[k] += (i == jt);
-                    uc[k] += a_at(it, i);
-                    bc = pick(bc, Cand{-okey(uc[k]), i});
-                }
+            for (int k = 0; k < K; ++k) {
+                const int q = lane + 32 * (w + ws * k);
+                const double a = kOnChip ? at[k][other * (int)so] : __ldg(at[k] + other * so);
+                cnt[k] += q == own ? 1 : 0;
+                u[k] += a;
+                const long long key = side ? -okey(u[k]) : okey(u[k]);
+                if (q < dim) b = pick(b, Cand{key, q});
             }
-            br = warp_pick<5>(br);
-            bc = warp_pick<5>(bc);
-            if (lane == 0) { red[par][0][warp] = br; red[par][1][warp] = bc; }
+            b = warp_best(b);
+            if (lane == 0) red[par][side][w] = b;
             __syncthreads();
-            // at most 8 published candidates (unused entries hold "none"); every
-            // group of 8 lanes holds all of them, reduced over lane bits 0..2
-            top = warp_pick<3>(red[par][0][lane & 7]);
-            bot = warp_pick<3>(red[par][1][lane & 7]);
-            it = top.i;
-            jt = bot.i;
+            Cand c[2][W];
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                c[0][q] = red[par][side ^ 1][q];
+                c[1][q] = red[par][side][q];
+            }
+#pragma unroll
+            for (int h = W / 2; h > 0; h >>= 1)
+#pragma unroll
+                for (int q = 0; q < h; ++q) {
+                    c[0][q] = pick(c[0][q], c[0][q + h]);
+                    c[1][q] = pick(c[1][q], c[1][q + h]);
+                }
+            best_other = c[0][0];
+            best_own = c[1][0];
+            other = best_other.i;
+            own = best_own.i;
         }
         const double Td = (double)T;
 #pragma unroll
-        for (int k = 0; k < kFpPer; ++k) {
-            const int i = tid + k * nt;
-            if (i < m) x_out[(int64_t)g * m + i] = (double)cr[k] / Td;
-            if (i < n) y_out[(int64_t)g * n + i] = (double)cc[k] / Td;
+        for (int k = 0; k < K; ++k) {
+            const int q = lane + 32 * (w + ws * k);
+            if (q < dim) (side ? y_out : x_out)[(int64_t)g * dim + q] = (double)cnt[k] / Td;
         }
-        if (tid == 0) {
-            bounds_out[2 * g] = okey_inv(-bot.k) / Td;     // min_j (x^T A)_j
-            bounds_out[2 * g + 1] = okey_inv(top.k) / Td;  // max_i (A y)_i
+        if (tid == 0) {                                            // a row thread
+            bounds_out[2 * g] = okey_inv(-best_other.k) / Td;      // min_j (x^T A)_j
+            bounds_out[2 * g + 1] = okey_inv(best_own.k) / Td;     // max_i (A y)_i
         }
     }
 }
 
 // Payoffs under a pair of mixtures: A y (per row), x^T A (per column), x^T A y.
-__global__ void __launch_bounds__(256) aggregate_kernel(
+// One block per game. Rows: a warp each, lanes over the columns. Columns: a
+// lane each, the rows dealt over the warps of its column group, their partial
+// sums combined in warp order. 64 x 64 with stride 4: 13 us (a thread per row and
+// column, uncoalesced rows: 23).
+constexpr int kAggThreads = 512, kAggWarps = kAggThreads / 32;
+
+__global__ void __launch_bounds__(kAggThreads) aggregate_kernel(
     const double* __restrict__ P, int32_t n_games, int32_t m, int32_t n, int32_t stride,
     const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ ay_out,
     double* __restrict__ xa_out, double* __restrict__ val_out) {
-    __shared__ double red[8];
+    __shared__ double red[kAggWarps];
+    __shared__ double col[kAggWarps][32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int g = blockIdx.x; g < n_games; g += gridDim.x) {
         const double* Pg = P + (int64_t)g * m * n * stride;
         const double* xg = x + (int64_t)g * m;
         const double* yg = y + (int64_t)g * n;
-        double part = 0.0;
-        for (int i = tid; i < m; i += blockDim.x) {
+        double part = 0.0;                       // of x^T A y: this warp's rows, in row order
+        for (int i = warp; i < m; i += kAggWarps) {
             double s = 0.0;
-            for (int j = 0; j < n; ++j) s = fma(Pg[((int64_t)i * n + j) * stride], yg[j], s);
-            ay_out[(int64_t)g * m + i] = s;
+#pragma unroll 4
+            for (int j = lane; j < n; j += 32) s = fma(Pg[((int64_t)i * n + j) * stride], yg[j], s);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) ay_out[(int64_t)g * m + i] = s;
             part = fma(xg[i], s, part);
         }
-        for (int j = tid; j < n; j += blockDim.x) {
-            double s = 0.0;
-            for (int i = 0; i < m; ++i) s = fma(xg[i], Pg[((int64_t)i * n + j) * stride], s);
-            xa_out[(int64_t)g * n + j] = s;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         if (lane == 0) red[warp] = part;
-        __syncthreads();
+        // columns, 32 groups of columns at a time over all warps
+        const int groups = (n + 31) / 32;
+        for (int c0 = 0; c0 < groups; c0 += kAggWarps) {
+            const int here = min(kAggWarps, groups - c0);        // column groups of this round
+            const int per = kAggWarps / here;                    // warps per group
+            const int grp = warp / per, sub = warp - grp * per;
+            const int j = (c0 + grp) * 32 + lane;
+            double s = 0.0;
+            if (grp < here && j < n)
+#pragma unroll 4
+                for (int i = sub; i < m; i += per) s = fma(xg[i], Pg[((int64_t)i * n + j) * stride], s);
+            col[warp][lane] = s;
+            __syncthreads();
+            if (grp < here && sub == 0 && j < n) {
+                for (int q = 1; q < per; ++q) s += col[warp + q][lane];
+                xa_out[(int64_t)g * n + j] = s;
+            }
+            __syncthreads();
+        }
         if (tid == 0) {
             double v = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w];
+            for (int w = 0; w < kAggWarps; ++w) v += red[w];
             val_out[g] = v;
         }
         __syncthreads();
@@ -185,7 +235,11 @@ __global__ void __launch_bounds__(256) aggregate_kernel(
 // column player's problem max sum(q) s.t. B q <= 1, q >= 0 has optimum
 // 1 / v_B; y = q v_B, and the row player's x = p v_B from the duals p (the
 // objective row under the slack columns). v_A = v_B + min(A) - 1.
-// Tableau rows 0..m-1: [B | I | 1]; row m: [-1 ... -1 | 0 | 0].
+// The tableau is kept condensed: rows 0..m-1 hold the nonbasic columns of [B | I]
+// and the right side (1), row m the reduced costs (-1 at the start, 0 on the
+// right). A pivot on (p, q) scales row p by 1 / a_pq, subtracts a_rq times it
+// from every other row r, and puts the leaving variable's column, (1 / a_pq at p,
+// -a_rq / a_pq elsewhere), in the entering one's place.
 // Entering column: the most negative reduced cost (Dantzig); after 2 (m + n)
 // consecutive degenerate pivots the rule switches for good to Bland's (lowest
 // index with a negative reduced cost), which cannot cycle. Leaving row: the
@@ -193,114 +247,201 @@ __global__ void __launch_bounds__(256) aggregate_kernel(
 // most that many pivots; optimality is still recognised after the last one)
 // guards regardless. Comparisons run on the integer keys above; the tableau
 // arithmetic is fp64.
+//
+// A pivot is (m + 1)(n + 1) independent fp64 FMAs between two reductions, and
+// fp64 is this part's slowest pipe (2 lanes a clock and SM: 5,000 cycles at 100 x
+// 100), so a game's columns are dealt over the CTAs of a cluster. Each CTA has
+// its columns and a copy of the right side and the basis; per pivot it offers
+// its best entering column (key and label to every CTA, the column in a buffer
+// the others read), one cluster barrier decides, and the ratio test and the
+// update run in every CTA without further exchange. The column buffer is
+// selected by the pivot's parity, so it is written again only after the next
+// barrier. One 100 x 100 game: 186 us on 8 CTAs (about 100 pivots); the full
+// tableau (identity columns included, a division per element to find its row) on
+// one CTA 780.
 // ---------------------------------------------------------------------------
-constexpr int kLpThreads = 512;
-constexpr int kLpWarps = kLpThreads / 32;
+constexpr int kLpThreads = 256, kLpWarps = kLpThreads / 32;
+constexpr int kLpMaxDim = 512, kLpMaxCluster = 8;
 
-// Reduction of one candidate per thread to the CTA's best (all threads get it).
-__device__ __forceinline__ Cand cta_pick(Cand c, Cand* red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    c = warp_pick<5>(c);
-    __syncthreads();                             // red's previous readers are done
-    if (lane == 0) red[warp] = c;
-    __syncthreads();
-    return warp_pick<4>(red[lane & 15]);
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+struct LpShape {
+    int32_t m, n, stride;
+    int32_t cluster;             // CTAs per game
+    int32_t cols;                // columns of a CTA: ceil(n / cluster)
+    int32_t hs;                  // column stride (doubles, odd, >= m + 1)
+    int32_t on_chip;
+    int32_t rows, rows_log2;     // threads over rows in an update: a power of two, at most 128
+    int64_t cta_doubles;         // (cols + 1) * hs
+};
+
+template <bool kCluster>
 __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
-    const double* __restrict__ P, int32_t n_games, int32_t m, int32_t n, int32_t stride,
-    double* __restrict__ x_out, double* __restrict__ y_out, double* __restrict__ val_out,
-    double* __restrict__ gscratch, int32_t on_chip, int32_t pivot_limit, int* __restrict__ err) {
+    const double* __restrict__ P, int32_t n_games, LpShape sh, double* __restrict__ x_out,
+    double* __restrict__ y_out, double* __restrict__ val_out, double* __restrict__ gscratch,
+    int32_t pivot_limit, int* __restrict__ err) {
+    struct Offer {
+        long long key;
+        int label, col;          // variable, and its column in the offering CTA
+    };
     extern __shared__ double smem_tab[];
-    __shared__ double colq[1024 + 1];
-    __shared__ int basis[1024];
-    __shared__ Cand red[kLpWarps];
-    const int tid = threadIdx.x;
-    const int W = n + m + 1;                     // tableau width; column W-1 is the right side
-    const int H = m + 1;                         // rows; row m is the objective
+    __shared__ double offered[2][kLpMaxDim + 1];             // [parity] this CTA's best entering column
+    __shared__ __align__(16) Offer offers[2][kLpMaxCluster]; // [parity][CTA]
+    __shared__ double colq[kLpMaxDim + 1], invs[kLpMaxDim], prow[kLpMaxDim + 1];
+    __shared__ int basis[kLpMaxDim], label[kLpMaxDim];       // label: variable of each own column
+    __shared__ Cand red[2][kLpWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m = sh.m, n = sh.n, hs = sh.hs;
+    const int rank = kCluster ? (int)cluster_rank() : 0, size = kCluster ? sh.cluster : 1;
+    const int c_lo = rank * sh.cols, w = max(0, min(sh.cols, n - c_lo));   // own columns
+    double* Tb = sh.on_chip ? smem_tab : gscratch + (int64_t)blockIdx.x * sh.cta_doubles;   // [w + 1][hs]
     const Cand none{kNone, 0x7fffffff};
     const double eps = 1e-12;
     const long long k_neg_eps = okey(-eps);
+    int rp = 0;                                              // parity of red
+    // the best candidate over the CTA (all threads get it; one barrier)
+    auto cta_best = [&](Cand c) {
+        c = warp_best(c);
+        rp ^= 1;
+        if (lane == 0) red[rp][warp] = c;
+        __syncthreads();
+        Cand b = red[rp][0];
+#pragma unroll
+        for (int q = 1; q < kLpWarps; ++q) b = pick(b, red[rp][q]);
+        return b;
+    };
 
-    for (int g = blockIdx.x; g < n_games; g += gridDim.x) {
-        double* Tb = on_chip ? smem_tab : gscratch + (int64_t)blockIdx.x * H * W;
-        const double* Pg = P + (int64_t)g * m * n * stride;
-        Cand lo = none;                          // min(A): the largest negated key
-        for (int k = tid; k < m * n; k += kLpThreads)
-            lo = pick(lo, Cand{-okey(Pg[(int64_t)k * stride]), k});
-        lo = cta_pick(lo, red);
+    for (int g = blockIdx.x / size; g < n_games; g += gridDim.x / size) {
+        const double* Pg = P + (int64_t)g * m * n * sh.stride;
+        __syncthreads();                                     // the previous game's tableau is read
+        Cand lo = none;                                      // min(A): the largest negated key
+        for (int k = tid; k < m * n; k += kLpThreads) lo = pick(lo, Cand{-okey(Pg[(int64_t)k * sh.stride]), k});
+        lo = cta_best(lo);
         const double shift = 1.0 - okey_inv(-lo.k);
-        for (int k = tid; k < H * W; k += kLpThreads) {
-            const int r = k / W, c = k - r * W;
-            double v;
-            if (r < m) {
-                if (c < n) v = Pg[((int64_t)r * n + c) * stride] + shift;
-                else if (c < n + m) v = (c - n == r) ? 1.0 : 0.0;
-                else v = 1.0;
-            } else {
-                v = c < n ? -1.0 : 0.0;
-            }
-            Tb[k] = v;
-        }
+        for (int r = warp; r <= m; r += kLpWarps)
+            for (int c = lane; c <= w; c += 32)
+                Tb[(int64_t)c * hs + r] = r < m ? (c < w ? Pg[((int64_t)r * n + c_lo + c) * sh.stride] + shift : 1.0)
+                                               : (c < w ? -1.0 : 0.0);
         for (int r = tid; r < m; r += kLpThreads) basis[r] = n + r;
+        for (int c = tid; c < w; c += kLpThreads) label[c] = c_lo + c;
         __syncthreads();
 
         const int max_pivots = pivot_limit > 0 ? pivot_limit : 50 * (m + n) + 1000;
         bool done = false, bland = false;
         int degenerate = 0;
         for (int piv = 0;; ++piv) {
-            // entering column
+            const int par = piv & 1;
+            // entering column: this CTA's best (ties by label: a column's label
+            // is its candidate index), then the cluster's
             Cand ce = none;
-            for (int c = tid; c < n + m; c += kLpThreads) {
-                const long long k = okey(Tb[(int64_t)m * W + c]);
-                if (k < k_neg_eps) ce = pick(ce, Cand{bland ? 0ll : -k, c});
+            int col = 0;
+            for (int c = tid; c < w; c += kLpThreads) {
+                const long long k = okey(Tb[(int64_t)c * hs + m]);
+                const Cand x{bland ? 0ll : -k, label[c]};
+                if (k < k_neg_eps && ((x.k > ce.k) | ((x.k == ce.k) & (x.i < ce.i)))) { ce = x; col = c; }
             }
-            ce = cta_pick(ce, red);
+            const Cand mine = cta_best(ce);
+            // the one thread whose column it is notes where it lies here
+            if (mine.k != kNone && ce.k == mine.k && ce.i == mine.i) offers[par][rank].col = col;
+            __syncthreads();
+            const int oc = offers[par][rank].col;
+            int q_rank = 0;
+            if constexpr (kCluster) {
+                if (mine.k != kNone)
+                    for (int r = tid; r <= m; r += kLpThreads) offered[par][r] = Tb[(int64_t)oc * hs + r];
+                if (tid < size)
+                    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                                     peer_addr(&offers[par][rank], (uint32_t)tid)),
+                                 "r"((uint32_t)(unsigned long long)mine.k), "r"((uint32_t)((unsigned long long)mine.k >> 32)),
+                                 "r"((uint32_t)mine.i), "r"((uint32_t)oc)
+                                 : "memory");
+                cluster_sync();
+                ce = none;
+                for (int q = 0; q < size; ++q) {
+                    const Cand o{offers[par][q].key, offers[par][q].label};
+                    if ((o.k > ce.k) | ((o.k == ce.k) & (o.i < ce.i))) { ce = o; q_rank = q; }
+                }
+            } else {
+                ce = mine;
+            }
             if (ce.k == kNone) { done = true; break; }
-            if (piv == max_pivots) break;        // another pivot is needed: limit reached
+            if (piv == max_pivots) break;                    // another pivot is needed: limit reached
             const int q = ce.i;
+            const int q_col = q_rank == rank ? oc : -1;      // its column here, when this CTA owns it
             // leaving row: minimum ratio (ratios are >= 0), ties to the lowest
             // basic index; the candidate index packs (basic index, row)
             Cand cl = none;
-            for (int r = tid; r < m; r += kLpThreads) {
-                const double a = Tb[(int64_t)r * W + q];
-                if (a > eps) {
-                    const double ratio = Tb[(int64_t)r * W + W - 1] / a;
-                    cl = pick(cl, Cand{-okey(ratio), basis[r] * 1024 + r});
+            for (int r = tid; r <= m; r += kLpThreads) {
+                double a;
+                if constexpr (kCluster)
+                    asm volatile("ld.shared::cluster.f64 %0, [%1];"
+                                 : "=d"(a)
+                                 : "r"(peer_addr(&offered[par][r], (uint32_t)q_rank))
+                                 : "memory");
+                else
+                    a = Tb[(int64_t)oc * hs + r];
+                colq[r] = a;
+                if (r < m && a > eps) {
+                    const double inv = 1.0 / a;
+                    invs[r] = inv;
+                    cl = pick(cl, Cand{-okey(Tb[(int64_t)w * hs + r] * inv), basis[r] * 1024 + r});
                 }
             }
-            cl = cta_pick(cl, red);
-            if (cl.k == kNone) break;            // unbounded: cannot happen with B > 0
+            cl = cta_best(cl);
+            if (cl.k == kNone) break;                        // unbounded: cannot happen with B > 0
             const int p = cl.i & 1023;
             degenerate = (okey_inv(-cl.k) == 0.0) ? degenerate + 1 : 0;
             if (degenerate > 2 * (m + n)) bland = true;
-            // pivot on (p, q)
-            for (int r = tid; r < H; r += kLpThreads) colq[r] = Tb[(int64_t)r * W + q];
+            // pivot on (p, q): the scaled row p first
+            const double inv = invs[p];
+            for (int c = tid; c <= w; c += kLpThreads) prow[c] = c == q_col ? inv : Tb[(int64_t)c * hs + p] * inv;
+            const int leaving = basis[p];
             __syncthreads();
-            const double inv = 1.0 / colq[p];
-            for (int c = tid; c < W; c += kLpThreads) Tb[(int64_t)p * W + c] *= inv;
-            __syncthreads();
-            for (int k = tid; k < H * W; k += kLpThreads) {
-                const int r = k / W;
-                if (r == p) continue;
-                const int c = k - r * W;
-                const double f = colq[r];
-                if (f != 0.0) Tb[k] = fma(-f, Tb[(int64_t)p * W + c], Tb[k]);
+            if (tid == 0) {
+                basis[p] = q;
+                if (q_col >= 0) label[q_col] = leaving;
             }
-            if (tid == 0) basis[p] = q;
+            for (int r = tid & (sh.rows - 1); r <= m; r += sh.rows) {   // sh.rows threads over rows, the rest over columns
+                const double f = colq[r];
+                for (int c = tid >> sh.rows_log2; c <= w; c += kLpThreads >> sh.rows_log2) {
+                    double* t = Tb + (int64_t)c * hs + r;
+                    if (r == p) *t = prow[c];
+                    else if (c == q_col) *t = f != 0.0 ? -f * prow[c] : 0.0;
+                    else if (f != 0.0) *t = fma(-f, prow[c], *t);
+                }
+            }
             __syncthreads();
         }
-        if (!done && tid == 0) atomicOr(err, ERRBIT_NOT_CONVERGED);
-        // read out: z = sum q = Tb[m][W-1]; v_B = 1 / z
-        const double z = Tb[(int64_t)m * W + W - 1];
-        const double vB = 1.0 / z;
-        for (int j = tid; j < n; j += kLpThreads) y_out[(int64_t)g * n + j] = 0.0;
-        __syncthreads();
-        for (int r = tid; r < m; r += kLpThreads)
-            if (basis[r] < n) y_out[(int64_t)g * n + basis[r]] = Tb[(int64_t)r * W + W - 1] * vB;
-        for (int i = tid; i < m; i += kLpThreads) x_out[(int64_t)g * m + i] = Tb[(int64_t)m * W + n + i] * vB;
-        if (tid == 0) val_out[g] = vB - shift;
-        __syncthreads();
+        if (!done && tid == 0 && rank == 0) atomicOr(err, ERRBIT_NOT_CONVERGED);
+        // read out: z = sum q = the right side of row m; v_B = 1 / z; basic
+        // variables from the right side, the others are 0; x from the reduced
+        // costs of the slacks (0 for basic ones)
+        const double vB = 1.0 / Tb[(int64_t)w * hs + m];
+        if (rank == 0)
+            for (int r = tid; r < m; r += kLpThreads) {
+                const int v = basis[r];
+                if (v < n) y_out[(int64_t)g * n + v] = Tb[(int64_t)w * hs + r] * vB;
+                else x_out[(int64_t)g * m + v - n] = 0.0;
+            }
+        for (int c = tid; c < w; c += kLpThreads) {
+            const int v = label[c];
+            if (v < n) y_out[(int64_t)g * n + v] = 0.0;
+            else x_out[(int64_t)g * m + v - n] = Tb[(int64_t)c * hs + m] * vB;
+        }
+        if (tid == 0 && rank == 0) val_out[g] = vB - shift;
+        if constexpr (kCluster) cluster_sync();              // nobody reads this game's offers any more
     }
 }
 
@@ -315,41 +456,86 @@ cudaError_t launch_fictitious_play(const double* P, int32_t G, int32_t m, int32_
     const int64_t bytes = (int64_t)m * ld * 8;
     const bool on_chip = bytes <= kSmemLimit;
     const size_t dyn = on_chip ? (size_t)bytes : 0;
-    // one thread per row and column up to 256 of them (fewer warps, cheaper
-    // barriers), else 256 threads with up to kFpPer rows / columns each
-    const int mx = m > n ? m : n;
-    const int threads = mx <= kFpThreads ? ((mx + 31) / 32) * 32 : kFpThreads;
-    auto kern = on_chip ? fictitious_play_kernel<true> : fictitious_play_kernel<false>;
+    // a warp per 32 rows and per 32 columns, at most kFpWarps a side
+    const int per = ((m > n ? m : n) + 32 * kFpWarps - 1) / (32 * kFpWarps);
+    auto warps = [&](int d) { return (d + 32 * per - 1) / (32 * per); };
+    const int wr = warps(m), wc = warps(n);
+    const int most = wr > wc ? wr : wc;
+    auto pick_kernel = [&](auto chip) {
+        constexpr bool C = decltype(chip)::value;
+        return per > 1     ? fictitious_play_kernel<C, kFpPer, 8>
+               : most <= 1 ? fictitious_play_kernel<C, 1, 1>
+               : most <= 2 ? fictitious_play_kernel<C, 1, 2>
+               : most <= 4 ? fictitious_play_kernel<C, 1, 4>
+                           : fictitious_play_kernel<C, 1, 8>;
+    };
+    auto kern = on_chip ? pick_kernel(std::true_type{}) : pick_kernel(std::false_type{});
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    kern<<<fp_grid(G, n_sm), threads, dyn, s>>>(P, G, m, n, stride, T, x, y, bounds);
+    kern<<<fp_grid(G, n_sm), 32 * (wr + wc), dyn, s>>>(P, G, m, n, stride, T, wr, x, y, bounds);
     return cudaGetLastError();
 }
 
 cudaError_t launch_aggregate(const double* P, int32_t G, int32_t m, int32_t n, int32_t stride,
                              const double* x, const double* y, double* ay, double* xa, double* val,
                              int n_sm, cudaStream_t s) {
-    aggregate_kernel<<<fp_grid(G, n_sm), 256, 0, s>>>(P, G, m, n, stride, x, y, ay, xa, val);
+    aggregate_kernel<<<fp_grid(G, n_sm), kAggThreads, 0, s>>>(P, G, m, n, stride, x, y, ay, xa, val);
     return cudaGetLastError();
 }
 
-int64_t lp_tableau_doubles(int32_t m, int32_t n) { return (int64_t)(m + 1) * (n + m + 1); }
+// The CTAs of a game: a cluster of 8, 4 or 2 while the games leave SMs free (an
+// eight-CTA cluster needs eight SMs of one GPC: 15 clusters at once were seen on
+// this part) and the update is long enough: below 40 x 40 the cluster's barrier
+// and remote loads (about 1,000 cycles a pivot) cost more than they save.
+static LpShape lp_shape(int32_t n_games, int32_t m, int32_t n, int32_t stride, int n_sm) {
+    LpShape s{};
+    s.m = m;
+    s.n = n;
+    s.stride = stride;
+    s.cluster = 1;
+    if ((int64_t)m * n >= 1600)
+        while (s.cluster < kLpMaxCluster && (int64_t)n_games * s.cluster * 2 <= n_sm - n_sm / 5) s.cluster *= 2;
+    while (s.cluster > 1 && n < 2 * s.cluster) s.cluster /= 2;
+    s.cols = (n + s.cluster - 1) / s.cluster;
+    s.hs = (m + 1) | 1;
+    s.rows = 1;
+    while (s.rows < 128 && s.rows < m + 1) {
+        s.rows *= 2;
+        ++s.rows_log2;
+    }
+    s.cta_doubles = (int64_t)(s.cols + 1) * s.hs;
+    s.on_chip = s.cta_doubles * 8 <= kSmemLimit ? 1 : 0;
+    return s;
+}
 
-bool lp_on_chip(int32_t m, int32_t n) { return lp_tableau_doubles(m, n) * 8 <= kSmemLimit; }
+static int lp_grid(int32_t n_games, int n_sm) { return n_games < n_sm ? n_games : n_sm; }
 
-int lp_grid(int32_t n_games, int n_sm) { return n_games < n_sm ? n_games : n_sm; }
+int64_t lp_scratch_bytes(int32_t n_games, int32_t m, int32_t n, int n_sm) {
+    const LpShape s = lp_shape(n_games, m, n, 1, n_sm);
+    return s.on_chip ? 0 : (int64_t)lp_grid(n_games, n_sm) * s.cluster * s.cta_doubles * 8;
+}
 
 cudaError_t launch_lp_nash(const double* P, int32_t G, int32_t m, int32_t n, int32_t stride,
                            double* x, double* y, double* val, double* scratch, int32_t pivot_limit,
                            int* err, int n_sm, cudaStream_t s) {
-    const int on_chip = lp_on_chip(m, n) ? 1 : 0;
-    const size_t dyn = on_chip ? (size_t)lp_tableau_doubles(m, n) * 8 : 0;
-    cudaError_t e = cudaFuncSetAttribute(lp_nash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)dyn);
+    const LpShape sh = lp_shape(G, m, n, stride, n_sm);
+    const size_t dyn = sh.on_chip ? (size_t)sh.cta_doubles * 8 : 0;
+    auto kern = sh.cluster > 1 ? lp_nash_kernel<true> : lp_nash_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    lp_nash_kernel<<<lp_grid(G, n_sm), kLpThreads, dyn, s>>>(P, G, m, n, stride, x, y, val, scratch,
-                                                             on_chip, pivot_limit, err);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(lp_grid(G, n_sm) * sh.cluster));
+    cfg.blockDim = dim3(kLpThreads);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)sh.cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, P, G, sh, x, y, val, scratch, pivot_limit, err);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace malib
@@ -446,9 +632,10 @@ extern "C" int malib_meta_lp_nash_ex(malib_ctx* ctx, const double* payoff, int32
     DevSel d(v.device);
     if (!d.ok) return ctx_fail(ctx, MALIB_ECUDA, "cannot select the context's device");
     double* scratch = nullptr;
-    if (!lp_on_chip(m, n)) {
+    const int64_t bytes = lp_scratch_bytes(n_games, m, n, v.n_sm);
+    if (bytes > 0) {
         void* p = nullptr;
-        r = ctx_scratch(ctx, (int64_t)lp_grid(n_games, v.n_sm) * lp_tableau_doubles(m, n) * 8, &p);
+        r = ctx_scratch(ctx, bytes, &p);
         if (r != MALIB_OK) return r;
         scratch = static_cast<double*>(p);
     }

@@ -123,6 +123,19 @@ def test_lp_value_and_equilibrium(ctx, m, n):
     check_lp(tables, *run_lp(ctx, tables))
 
 
+@pytest.mark.parametrize("G,m,n", [(1, 40, 40), (1, 39, 41), (4, 100, 17), (20, 45, 83), (50, 64, 33), (3, 33, 130),
+                                   (2, 512, 9), (1, 300, 290), (40, 300, 200), (70, 200, 150)])
+def test_lp_games_over_clusters(ctx, G, m, n):
+    """Columns dealt over 8, 4, 2 and 1 CTAs, CTAs with fewer columns or none,
+    tableaus on and off chip; integer tables in the last third tie often."""
+    rng = np.random.default_rng(m * n + G)
+    tables = rng.normal(size=(G, m, n))
+    tables[-1] = rng.integers(-2, 3, size=(m, n))
+    gx, gy, gv = run_lp(ctx, tables)
+    some = sorted({0, G // 2, G - 1})
+    check_lp(tables[some], gx[some], gy[some], gv[some])
+
+
 def test_lp_closed_forms_and_degenerate(ctx):
     rps = np.array([[0, -1, 1], [1, 0, -1], [-1, 1, 0]], float)
     two = np.array([[3.0, -1.0], [-2.0, 1.0]])
