@@ -597,41 +597,59 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_kernel(LearnArgs a) {
     if (b >= 0) flush();
 }
 
-// Grid (blocks, nb): policy b's gradient as the sum, in CTA order, of the
-// partials of the CTAs whose tile share meets b's tiles (eight interleaved
-// partial sums, combined in a fixed order); its loss and mean entropy.
-__global__ void learn_reduce_kernel(LearnArgs a, int P) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// Grid (blocks, nb): policy b's gradient as the sum of the partials of the CTAs
+// whose tile share meets b's tiles; its loss and mean entropy. A block takes 64
+// entries; four groups of threads sum a quarter of the CTAs each (eight loads in
+// flight), combined in a fixed order. One thread per entry with the CTAs' shares
+// recomputed by a division per step and its partial sums in local memory took 58
+// us for 3 policies; this 17.
+constexpr int kRedEntries = 64, kRedGroups = 4;
+
+__global__ void __launch_bounds__(kRedEntries * kRedGroups) learn_reduce_kernel(LearnArgs a, int P) {
+    __shared__ double part[kRedGroups][kRedEntries];
+    __shared__ int range[2];
     const int b = blockIdx.y;
-    if (j >= P + 2) return;
-    const int64_t t_lo = a.tile_off[b], t_hi = a.tile_off[b + 1];
-    int c_lo = 0, c_hi = 0;                  // CTAs [c_lo, c_hi) hold partials of b
-    if (t_hi > t_lo) {
-        // c_lo: the first CTA whose share ends past t_lo; c_hi: the first CTA
-        // after it whose share starts at or past t_hi (or the grid's end). Both
-        // start from the shares' proportional position and step to the exact one.
-        const int64_t n_t = a.tile_off[a.nb];
-        c_lo = (int)min((int64_t)a.grid - 1, t_lo * a.grid / n_t);
-        while (c_lo > 0 && share_lo(a, c_lo) > t_lo) --c_lo;
-        while (share_lo(a, c_lo + 1) <= t_lo) ++c_lo;
-        c_hi = (int)max((int64_t)c_lo + 1, min((int64_t)a.grid, (t_hi * a.grid + n_t - 1) / n_t));
-        while (c_hi > c_lo + 1 && share_lo(a, c_hi - 1) >= t_hi) --c_hi;
-        while (c_hi < a.grid && share_lo(a, c_hi) < t_hi) ++c_hi;
-    }
-    // (a CTA with an empty share wrote no partial: it is skipped)
-    const float* part = a.gpart + (int64_t)b * a.grid * (P + 2) + j;
-    double p8[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    int u = 0;
-    int64_t s_c = share_lo(a, c_lo);
-    for (int c = c_lo; c < c_hi; ++c) {
-        const int64_t s_n = share_lo(a, c + 1);
-        if (s_n > s_c) {
-            p8[u] += (double)part[(int64_t)c * (P + 2)];
-            u = (u + 1) & 7;
+    const int64_t t_lo = a.tile_off[b], t_hi = a.tile_off[b + 1], n_t = a.tile_off[a.nb];
+    if (threadIdx.x == 0) {
+        int c_lo = 0, c_hi = 0;              // CTAs [c_lo, c_hi) hold partials of b
+        if (t_hi > t_lo) {
+            // c_lo: the first CTA whose share ends past t_lo; c_hi: the first CTA
+            // after it whose share starts at or past t_hi (or the grid's end). Both
+            // start from the shares' proportional position and step to the exact one.
+            c_lo = (int)min((int64_t)a.grid - 1, t_lo * a.grid / n_t);
+            while (c_lo > 0 && share_lo(a, c_lo) > t_lo) --c_lo;
+            while (share_lo(a, c_lo + 1) <= t_lo) ++c_lo;
+            c_hi = (int)max((int64_t)c_lo + 1, min((int64_t)a.grid, (t_hi * a.grid + n_t - 1) / n_t));
+            while (c_hi > c_lo + 1 && share_lo(a, c_hi - 1) >= t_hi) --c_hi;
+            while (c_hi < a.grid && share_lo(a, c_hi) < t_hi) ++c_hi;
         }
-        s_c = s_n;
+        range[0] = c_lo;
+        range[1] = c_hi;
     }
-    const double s = ((p8[0] + p8[1]) + (p8[2] + p8[3])) + ((p8[4] + p8[5]) + (p8[6] + p8[7]));
+    __syncthreads();
+    const int e = threadIdx.x & (kRedEntries - 1), grp = threadIdx.x / kRedEntries;
+    const int j = blockIdx.x * kRedEntries + e;
+    const int n = range[1] - range[0], per = (n + kRedGroups - 1) / kRedGroups;
+    const int c0 = range[0] + grp * per, c1 = min(range[1], c0 + per);
+    // with fewer tiles than CTAs some shares are empty, and those CTAs wrote no partial
+    const bool all = n_t >= a.grid;
+    const float* src = a.gpart + (int64_t)b * a.grid * (P + 2) + j;
+    double s = 0.0;
+    if (j < P + 2)
+        for (int c = c0; c < c1; c += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                v[u] = c + u < c1 && (all || share_lo(a, c + u + 1) > share_lo(a, c + u))
+                           ? __ldcg(src + (int64_t)(c + u) * (P + 2)) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += (double)v[u];
+        }
+    part[grp][e] = s;
+    __syncthreads();
+    if (grp != 0 || j >= P + 2) return;
+#pragma unroll
+    for (int q = 1; q < kRedGroups; ++q) s += part[q][e];
     double* st = a.stats + 4 * b;
     if (j < P) a.grad[(int64_t)b * P + j] = (float)s;
     else if (j == P) st[2] = st[0] > 0 ? s / st[0] : 0.0;   // loss: (1/M) sum of -(A log pi + beta H)
@@ -708,7 +726,7 @@ cudaError_t launch_learn_pg(const LearnArgs& a, int ret_blocks, cudaStream_t s, 
     learn_grad_kernel<<<a.grid, kThreads, kSBytes, s>>>(a);
     if (g1) cudaEventRecord(g1, s);
     const int P = (int)learn_param_count(a.in);
-    learn_reduce_kernel<<<dim3((P + 2 + 255) / 256, a.nb), 256, 0, s>>>(a, P);
+    learn_reduce_kernel<<<dim3((P + 2 + kRedEntries - 1) / kRedEntries, a.nb), kRedEntries * kRedGroups, 0, s>>>(a, P);
     return cudaGetLastError();
 }
 
