@@ -194,6 +194,8 @@ struct ConvJob {
 };
 cudaError_t launch_pop_convert(const ConvJob* jobs, int n_jobs, int64_t max_size, const float* stage,
                                float* arena, cudaStream_t s);
+// The same for one policy whose plain parameters are at src (device memory).
+cudaError_t launch_pop_convert_one(const ConvJob& job, const float* src, float* arena, cudaStream_t s);
 
 cudaError_t launch_philox_digest(uint64_t seed, int64_t n, int calls, uint32_t* out,
                                  cudaStream_t s);

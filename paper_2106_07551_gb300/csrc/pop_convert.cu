@@ -113,10 +113,7 @@ __device__ uint32_t tc_word(const float* p, const int* d, bool fold, int64_t i) 
     return h[0] | (h[1] << 16);
 }
 
-__global__ void pop_convert_kernel(const ConvJob* __restrict__ jobs, const float* __restrict__ stage,
-                                   float* __restrict__ arena) {
-    const ConvJob j = jobs[blockIdx.y];
-    const float* src = stage + j.src;
+__device__ __forceinline__ void convert(const ConvJob& j, const float* src, float* arena) {
     uint32_t* dst = reinterpret_cast<uint32_t*>(arena + j.dst);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < j.size;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -128,6 +125,18 @@ __global__ void pop_convert_kernel(const ConvJob* __restrict__ jobs, const float
     }
 }
 
+__global__ void pop_convert_kernel(const ConvJob* __restrict__ jobs, const float* __restrict__ stage,
+                                   float* __restrict__ arena) {
+    const ConvJob j = jobs[blockIdx.y];
+    convert(j, stage + j.src, arena);
+}
+
+// One policy, its job as a kernel parameter and its parameters where they lie.
+__global__ void pop_convert_one_kernel(const __grid_constant__ ConvJob j, const float* __restrict__ src,
+                                       float* __restrict__ arena) {
+    convert(j, src, arena);
+}
+
 }  // namespace
 
 cudaError_t launch_pop_convert(const ConvJob* jobs, int n_jobs, int64_t max_size, const float* stage,
@@ -137,6 +146,12 @@ cudaError_t launch_pop_convert(const ConvJob* jobs, int n_jobs, int64_t max_size
     const int64_t bx = (max_size + 255) / 256;
     const unsigned gx = (unsigned)(bx < 64 ? (bx < 1 ? 1 : bx) : 64);
     pop_convert_kernel<<<dim3(gx, (unsigned)n_jobs), 256, 0, s>>>(jobs, stage, arena);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pop_convert_one(const ConvJob& job, const float* src, float* arena, cudaStream_t s) {
+    const int64_t bx = (job.size + 255) / 256;
+    pop_convert_one_kernel<<<(unsigned)(bx < 64 ? (bx < 1 ? 1 : bx) : 64), 256, 0, s>>>(job, src, arena);
     return cudaGetLastError();
 }
 

@@ -844,10 +844,13 @@ int learn_batch(malib_ctx* c, const malib_env_spec* spec, const int32_t* pair_id
             return r;
         a.grad = c->learn_grad;
     }
-    CK(cudaMemcpyAsync(const_cast<int32_t*>(a.pols), hid.data(), (size_t)nb * 4, cudaMemcpyHostToDevice,
-                       c->stream), "policy ids");
-    CK(cudaMemcpyAsync(const_cast<int64_t*>(a.pol_offs), hoff.data(), (size_t)nb * 8, cudaMemcpyHostToDevice,
-                       c->stream), "policy offsets");
+    // ids and offsets lie together in the work space: one copy
+    const size_t offs_at = (size_t)((const uint8_t*)a.pol_offs - (const uint8_t*)a.pols);
+    std::vector<uint8_t> head(offs_at + (size_t)nb * 8);
+    std::memcpy(head.data(), hid.data(), (size_t)nb * 4);
+    std::memcpy(head.data() + offs_at, hoff.data(), (size_t)nb * 8);
+    CK(cudaMemcpyAsync(const_cast<int32_t*>(a.pols), head.data(), head.size(), cudaMemcpyHostToDevice, c->stream),
+       "policy ids and offsets");
     a.arena = c->arena;
     a.in = in;
     a.xs = (spec->obs_dim + 3) / 4 * 4;
@@ -883,8 +886,7 @@ int learn_batch(malib_ctx* c, const malib_env_spec* spec, const int32_t* pair_id
         CK(cudaMemcpyAsync(stats_out, a.stats, (size_t)nb * 4 * 8,
                            sw == kPtrHere ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream),
            "statistics copy");
-    // the host vectors of ids and offsets are copied before they go out of scope
-    CK(cudaStreamSynchronize(c->stream), "learner step");
+    // waits for the stream, and so for the host buffer's copy, before it goes out of scope
     return read_device_errors(c);
 }
 
@@ -952,18 +954,21 @@ int malib_pop_update(malib_ctx* c, int32_t policy_id, const float* params, int64
     if (!params || nbytes != count * 4)
         return fail(c, MALIB_EINVAL, "params NULL or nbytes %lld != %lld", (long long)nbytes,
                     (long long)(count * 4));
-    if (ptr_where(params, c->device) == kPtrOther)
-        return fail(c, MALIB_EINVAL, "params live on another device than the context's");
+    const int where = ptr_where(params, c->device);
+    if (where == kPtrOther) return fail(c, MALIB_EINVAL, "params live on another device than the context's");
     ConvJob jb{};
     conv_job(c->spec.env_kind, rec.kind, rec.dtype, rec.dims, &jb);
     jb.src = 0;
     jb.dst = rec.offset;
-    int r;
-    if ((r = ensure(c, c->d_stage, c->stage_cap, (count + 3) / 4 * 4, "parameter staging")) != MALIB_OK) return r;
-    if ((r = ensure(c, c->d_jobs, c->jobs_cap, (int64_t)1, "conversion jobs")) != MALIB_OK) return r;
-    CK(cudaMemcpyAsync(c->d_stage, params, nbytes, cudaMemcpyDefault, c->stream), "parameter upload");
-    CK(cudaMemcpyAsync(c->d_jobs, &jb, sizeof jb, cudaMemcpyHostToDevice, c->stream), "conversion job");
-    CK(launch_pop_convert(c->d_jobs, 1, jb.size, c->d_stage, c->arena, c->stream), "population conversion kernel");
+    // device parameters (float-aligned) are read where they lie; others are staged
+    const float* src = params;
+    if (where != kPtrHere || ((uintptr_t)params & 3u) != 0) {
+        int r;
+        if ((r = ensure(c, c->d_stage, c->stage_cap, (count + 3) / 4 * 4, "parameter staging")) != MALIB_OK) return r;
+        CK(cudaMemcpyAsync(c->d_stage, params, nbytes, cudaMemcpyDefault, c->stream), "parameter upload");
+        src = c->d_stage;
+    }
+    CK(launch_pop_convert_one(jb, src, c->arena, c->stream), "population conversion kernel");
     c->launches += 1;
     // the caller may free or reuse its buffer once this returns
     CK(cudaStreamSynchronize(c->stream), "population update");
