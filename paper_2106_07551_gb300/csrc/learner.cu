@@ -24,12 +24,14 @@
 //     G_t = r_t + gamma G_{t+1}, one thread per (slot, episode, env), and
 //     per-block fp64 sums of G.
 //  3. learn_baseline_kernel: M and b = sum G / M in a fixed order (one block).
-//  4. learn_grad_kernel: persistent CTAs over tiles of 128 samples: forward
-//     (fp32 FMA, hidden 64), logits, softmax, dL/dz, the backward pass, and
-//     the weight gradients accumulated in registers over the CTA's tiles (each
-//     thread a 4 x 4 block of dW2 and a few entries of the rest); the tile's
-//     activations are stored feature-major in shared memory so that every
-//     product reads 16-byte vectors; each CTA writes its partial gradient.
+//  4. learn_grad_x3_kernel (learner_x3.cu; observations up to 20 wide) or
+//     learn_grad_kernel (up to 32): persistent CTAs over tiles of 128 samples:
+//     forward (fp32, hidden 64), logits, softmax, dL/dz, the backward pass, and
+//     the weight gradients, summed over the CTA's tiles; each CTA writes its
+//     partial gradient. learn_grad_kernel in fp32 FMAs:
+//     each thread keeps a 4 x 4 block of dW2 and a few entries of the rest in
+//     registers; the tile's activations are stored feature-major in shared
+//     memory so that every product reads 16-byte vectors.
 //  5. learn_reduce_kernel: the partials summed over CTAs in a fixed order into
 //     the gradient (the malib_policy_desc layout) and the loss statistics.
 // Deterministic: no atomics, every sum in a fixed order.
@@ -37,8 +39,8 @@
 #include <cmath>
 
 #include "device_common.cuh"
-#include "internal.h"
 #include "f32x2.cuh"
+#include "learner_common.cuh"
 
 namespace malib {
 
@@ -192,20 +194,6 @@ __global__ void learn_baseline_kernel(LearnArgs a, int n_blocks) {
     a.stats[4 * b + 1] = M > 0 ? s / M : 0.0;
 }
 
-// Sample s of the policy's sample order: (slot, episode, step, env) -> the
-// trajectory index of its (episode, step, env, agent).
-__device__ __forceinline__ int64_t sample_index(const LearnArgs& a, const int32_t* slots, int64_t s, int epp) {
-    const int r = (int)(s % epp);
-    const int64_t q = s / epp;                        // (slot, e, t)
-    const int t = (int)(q % a.T);
-    const int64_t q2 = q / a.T;
-    const int64_t e = q2 % a.n_episodes, slot = q2 / a.n_episodes;
-    const int ck = slots[slot];
-    const int c = ck / a.n_agents, ka = ck - c * a.n_agents;
-    const int64_t env = (int64_t)c * epp + r;
-    return ((e * a.T + t) * a.n_envs + env) * a.n_agents + ka;
-}
-
 // H_out[j][s] = relu(b[j] + sum_k W[k][j] H_in[k][s]) for this thread's 8
 // samples (8 sg ..) and 4 outputs (ng + 16 q): per k two 16-byte loads of H_in
 // (four sample pairs) and four weights, each duplicated into a pair, for 16
@@ -252,12 +240,6 @@ __device__ __forceinline__ void store_masked(float* __restrict__ o, const unsign
                                                 h0.z > 0.f ? v1.x : 0.f, h0.w > 0.f ? v1.y : 0.f);
     *reinterpret_cast<float4*>(o + 4) = make_float4(h1.x > 0.f ? v2.x : 0.f, h1.y > 0.f ? v2.y : 0.f,
                                                     h1.z > 0.f ? v3.x : 0.f, h1.w > 0.f ? v3.y : 0.f);
-}
-
-// A CTA's contiguous share [lo, hi) of the batch's tiles (all policies' tiles
-// in policy order).
-__device__ __forceinline__ int64_t share_lo(const LearnArgs& a, int64_t c) {
-    return a.tile_off[a.nb] * c / a.grid;
 }
 
 __global__ void __launch_bounds__(kThreads, 1) learn_grad_kernel(LearnArgs a) {
@@ -713,17 +695,23 @@ void learn_work_layout(uint8_t* base, int32_t nb, int32_t n_pairs, int32_t n_age
     a->grid = grid;
 }
 
+static cudaError_t launch_learn_grad_f32(const LearnArgs& a, cudaStream_t s) {
+    const cudaError_t err = cudaFuncSetAttribute(learn_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)kSBytes);
+    if (err != cudaSuccess) return err;
+    learn_grad_kernel<<<a.grid, kThreads, kSBytes, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_learn_pg(const LearnArgs& a, int ret_blocks, cudaStream_t s, cudaEvent_t g0, cudaEvent_t g1) {
     if (a.nb <= 0) return cudaSuccess;
     learn_slots_kernel<<<a.nb, 1024, 0, s>>>(a);
     learn_plan_kernel<<<1, 32, 0, s>>>(a);
     learn_returns_kernel<<<dim3(ret_blocks, a.nb), 256, 0, s>>>(a);
     learn_baseline_kernel<<<a.nb, 32, 0, s>>>(a, ret_blocks);
-    cudaError_t err = cudaFuncSetAttribute(learn_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kSBytes);
-    if (err != cudaSuccess) return err;
     if (g0) cudaEventRecord(g0, s);
-    learn_grad_kernel<<<a.grid, kThreads, kSBytes, s>>>(a);
+    cudaError_t err = a.in <= kLearnX3MaxIn ? launch_learn_grad_x3(a, s) : launch_learn_grad_f32(a, s);
+    if (err != cudaSuccess) return err;
     if (g1) cudaEventRecord(g1, s);
     const int P = (int)learn_param_count(a.in);
     learn_reduce_kernel<<<dim3((P + 2 + kRedEntries - 1) / kRedEntries, a.nb), kRedEntries * kRedGroups, 0, s>>>(a, P);

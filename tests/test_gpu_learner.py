@@ -370,3 +370,82 @@ def test_ppo_batch_with_an_idle_policy_and_push():
         np.testing.assert_allclose([st[row, 1], st[row, 3]], [b, ent], rtol=1e-5, atol=1e-7)
         check_grad(g[row], o, dims)
     ctx.close()
+
+
+def synthetic(in_dim, epp=37, n_pairs=3, n_eps=3, seed=0, shift=0):
+    """Samples of a 2-agent spread spec of the given observation width: policy 0 acts in all
+    slots but one. `shift` floats put the observations off a 16-byte boundary."""
+    torch = need_gpu()
+    w = workloads.spread(n_agents=2, n_envs=epp * n_pairs, pop=2, obs_dim=in_dim, episode_len=7,
+                         envs_per_pair=epp, with_bias=True, seed=seed)
+    w.pair_ids[:] = 0
+    w.pair_ids[1, 0] = 1
+    rng = np.random.default_rng(seed + 1)
+    shape = (n_eps, 7, w.n_envs, 2)
+    xs = (in_dim + 3) // 4 * 4
+    obs = rng.uniform(-1.5, 1.5, shape + (xs,)).astype(np.float32)
+    obs[..., in_dim:] = 7.0                              # the row's padding is not read as a feature
+    flat = torch.zeros(obs.size + shift, device="cuda")
+    flat[shift:] = torch.from_numpy(obs.reshape(-1))
+    tr = {"obs": obs, "action": rng.integers(0, 5, shape).astype(np.uint8),
+          "reward": -rng.uniform(0.5, 2.5, shape).astype(np.float32)}
+    traj = {"obs": flat[shift:].view(shape + (xs,)), "action": torch.from_numpy(tr["action"]).cuda(),
+            "reward": torch.from_numpy(tr["reward"]).cuda()}
+    return w, tr, traj
+
+
+@pytest.mark.parametrize("in_dim,epp,shift", [(10, 1, 0), (11, 37, 1), (12, 128, 0), (13, 60, 2), (16, 129, 0),
+                                              (17, 43, 3), (18, 300, 0), (20, 37, 1), (21, 37, 0), (32, 37, 1)])
+def test_gradient_at_every_padded_width(in_dim, epp, shift):
+    """The edges of the tensor-core kernel's input widths (12, 16, 20; push has 8) and the general kernel past
+    them, with envs per combination below, at and above a 128-sample tile."""
+    need_gpu()
+    w, tr, traj = synthetic(in_dim, epp, seed=in_dim, shift=shift)
+    ctx = context()
+    load_population(ctx, w)
+    for pid in (0, 1):
+        g, st = learn(ctx, w, spec_of(w), traj, 3, pid, 0.9, 0.01)
+        o, (M, b, loss, ent) = oracle_grad(w, tr, pid, 0.9, 0.01)
+        assert st[0] == M and M > 0
+        np.testing.assert_allclose([st[1], st[3]], [b, ent], rtol=1e-5, atol=1e-7)
+        check_grad(g, o, w.policies[pid].dims)
+    ctx.close()
+
+
+@pytest.mark.parametrize("in_dim", [18, 24])
+def test_relu_inputs_within_rounding_of_zero(in_dim):
+    """Hidden units whose input is the rounding error of one product (w x - w x in an fp32 FMA chain,
+    features 0 and 1 the same): both kernels take the chain's sign, which the oracle's gradient gets
+    here as the ReLU's mask."""
+    torch = need_gpu()
+    w, tr, traj = synthetic(in_dim, 128, seed=3)
+    tr["obs"][..., 1] = tr["obs"][..., 0]
+    traj["obs"].copy_(torch.from_numpy(tr["obs"]))
+    dims, tiny = w.policies[0].dims, np.arange(0, 64, 5)
+    W1, b1, W2, b2, W3, b3 = [a.astype(np.float32) for a in learner.unpack(w.policies[0].params, dims)]
+    W1[tiny] = 0.0
+    W1[tiny, 0] = np.random.default_rng(4).uniform(0.2, 0.9, len(tiny)).astype(np.float32)
+    W1[tiny, 1] = -W1[tiny, 0]
+    b1[tiny] = 0.0
+    w.policies[0].params = np.concatenate([a.ravel() for a in (W1, b1, W2, b2, W3, b3)]).astype(np.float32)
+    ctx = context()
+    load_population(ctx, w)
+    g, _ = learn(ctx, w, spec_of(w), traj, 3, 0, 0.9, 0.01)
+    obs, act, ret = learner.gather(tr, w.pair_ids, w.n_envs, 2, in_dim, 0, 0.9)
+    # the chain: fl(x w) by the first FMA, then fl(fl(x w) - x w), exact in fp64
+    prod = obs[:, :1] * W1[tiny, 0].astype(np.float64)
+    on = prod.astype(np.float32).astype(np.float64) - prod > 0
+    assert 0.2 < on.mean() < 0.8
+    W2d, W3d = W2.astype(np.float64), W3.astype(np.float64)
+    pre1 = obs @ W1.T.astype(np.float64) + b1
+    pre1[:, tiny] = 0.0
+    pre2 = np.maximum(pre1, 0) @ W2d.T + b2
+    logp = learner.log_softmax(np.maximum(pre2, 0) @ W3d.T + b3)
+    pi = np.exp(logp)
+    H = -(pi * logp).sum(1)
+    dz = ((ret - ret.mean())[:, None] * (pi - np.eye(5)[act]) + 0.01 * pi * (logp + H[:, None])) / len(ret)
+    d1 = ((dz @ W3d) * (pre2 > 0)) @ W2d
+    want = (d1[:, tiny] * on).T @ obs                    # dW1 rows of the tiny units
+    got = g[:64 * in_dim].reshape(64, in_dim)[tiny]
+    np.testing.assert_allclose(got, want, rtol=0, atol=1e-4 * np.abs(want).max())
+    ctx.close()
