@@ -106,6 +106,9 @@ struct RolloutArgs {
 };
 
 // Launchers (return cudaGetLastError() of the launch). `grid_hint` = SM count.
+// launch_kuhn_eval with fin_out set needs none of acc, n_dec and work cleared: it
+// writes the table and every pair's decision count (work[pair]) without adding.
+bool kuhn_counts_itself(int32_t n_pairs, int64_t n_episodes, int n_sm);
 cudaError_t launch_kuhn_eval(const EvalArgs& a, int n_sm, cudaStream_t s);
 cudaError_t launch_kuhn_exact(const EvalArgs& a, double* out, cudaStream_t s);
 cudaError_t launch_leduc_eval_f32(const EvalArgs& a, int hidden, int n_sm, cudaStream_t s);

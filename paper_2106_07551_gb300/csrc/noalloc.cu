@@ -109,12 +109,15 @@ extern "C" int malib_eval_payoff_noalloc(malib_ctx* ctx, const int32_t* pair_ids
         a.acc = scratch;
         a.n_dec = scratch + 2 * (int64_t)n_pairs;
         a.work = scratch + 2 * (int64_t)n_pairs + 1;
-        if ((e = launch_zero_u64(scratch, 3 * (int64_t)n_pairs + 1, v.stream)) == cudaSuccess)
+        const bool one = v.env_kind == MALIB_ENV_KUHN && kuhn_counts_itself(n_pairs, n_episodes, v.n_sm);
+        if (one) a.fin_out = payoff_out;
+        if (!one) e = launch_zero_u64(scratch, 3 * (int64_t)n_pairs + 1, v.stream);
+        if (e == cudaSuccess)
             e = v.env_kind == MALIB_ENV_KUHN ? launch_kuhn_eval(a, v.n_sm, v.stream)
                                              : launch_leduc_eval_f32(a, v.dims[1], v.n_sm, v.stream);
-        if (e == cudaSuccess) e = launch_finalize(scratch, n_pairs, n_episodes, payoff_out, v.stream);
+        if (e == cudaSuccess && !one) e = launch_finalize(scratch, n_pairs, n_episodes, payoff_out, v.stream);
         if (e != cudaSuccess) code = ctx_fail(ctx, MALIB_ECUDA, cudaGetErrorString(e));
-        else ctx_count_launches(ctx, 3);
+        else ctx_count_launches(ctx, one ? 1 : 3);
     }
     if (prev >= 0) cudaSetDevice(prev);
     return code;

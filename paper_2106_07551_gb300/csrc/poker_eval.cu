@@ -52,25 +52,22 @@ __device__ __forceinline__ KuhnHand kuhn_play(const float (&t0)[6], const float 
     return h;
 }
 
-__global__ void __launch_bounds__(256) kuhn_eval_kernel(EvalArgs a) {
-    const int pair = blockIdx.y;
-    const int p0 = a.pairs[2 * pair], p1 = a.pairs[2 * pair + 1];
-    const bool ok = pair_ok(a, p0, p1);
-    if (!ok && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(a.err, ERRBIT_BAD_PAIR);
+// A thread's share of a pair's hands: e0, e0 + stride, ...; adds the payoffs, their
+// squares and the decisions to s1, s2, nd and records the first n_dump hands.
+template <class Sum>
+__device__ __forceinline__ void kuhn_hands(const EvalArgs& a, int pair, int p0, int p1, int64_t e0, int64_t stride,
+                                           Sum& s1, Sum& s2, Sum& nd) {
     float t0[6], t1[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        t0[i] = ok ? a.arena[a.pol_offset[p0] + i] : 0.f;
-        t1[i] = ok ? a.arena[a.pol_offset[p1] + i] : 0.f;
+        t0[i] = a.arena[a.pol_offset[p0] + i];
+        t1[i] = a.arena[a.pol_offset[p1] + i];
     }
-    long long s1 = 0, s2 = 0, nd = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t n_play = ok ? a.n_episodes : 0;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n_play; e += stride) {
+    for (int64_t e = e0; e < a.n_episodes; e += stride) {
         const uint64_t g = (uint64_t)pair * (uint64_t)a.n_episodes + (uint64_t)e;
         const KuhnHand h = kuhn_play(t0, t1, g, a.seed);
         s1 += h.payoff;
-        s2 += (long long)h.payoff * h.payoff;
+        s2 += (Sum)(h.payoff * h.payoff);
         nd += h.n;
         if (e < a.n_dump) {
             const int64_t base = ((int64_t)pair * a.n_dump + e) * 3;
@@ -86,6 +83,17 @@ __global__ void __launch_bounds__(256) kuhn_eval_kernel(EvalArgs a) {
             }
         }
     }
+}
+
+__global__ void __launch_bounds__(256) kuhn_eval_kernel(EvalArgs a) {
+    const int pair = blockIdx.y;
+    const int p0 = a.pairs[2 * pair], p1 = a.pairs[2 * pair + 1];
+    const bool ok = pair_ok(a, p0, p1);
+    if (!ok && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(a.err, ERRBIT_BAD_PAIR);
+    long long s1 = 0, s2 = 0, nd = 0;
+    if (ok)
+        kuhn_hands(a, pair, p0, p1, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x,
+                   s1, s2, nd);
     block_add_sums(s1, s2, nd, a.acc + 2 * pair, a.n_dec);
     // the pair's last block to finish writes its table row (its sums are final:
     // every block fenced its additions before counting itself)
@@ -98,6 +106,63 @@ __global__ void __launch_bounds__(256) kuhn_eval_kernel(EvalArgs a) {
             finalize_pair(f1, f2, a.n_episodes, a.fin_out + 4 * (int64_t)pair);
         }
     }
+}
+
+// The same with a cluster per pair: the CTAs' sums (32-bit: at most 4
+// hands a thread) meet in the first one's shared memory, which writes the pair's row and its
+// decision count. No accumulators in global memory to clear, add to and count
+// blocks with: a table of 16 pairs x 10,000 hands is bound by latencies, and took
+// KUHNFIG.
+constexpr int kKuhnMaxThreads = 768, kKuhnMaxCluster = 8;
+
+__global__ void __launch_bounds__(kKuhnMaxThreads, 2) kuhn_cluster_kernel(EvalArgs a) {
+    __shared__ int warp_sums[3][32], cta_sums[kKuhnMaxCluster][4];
+    uint32_t rank, size;
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");        // this CTA runs
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+    const int pair = (int)(blockIdx.x / size), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p0 = a.pairs[2 * pair], p1 = a.pairs[2 * pair + 1];
+    const bool ok = pair_ok(a, p0, p1);
+    int s[3] = {0, 0, 0};
+    if (ok)
+        kuhn_hands(a, pair, p0, p1, (int64_t)(rank * blockDim.x + threadIdx.x), (int64_t)(size * blockDim.x), s[0], s[1], s[2]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int v = __reduce_add_sync(0xffffffffu, s[i]);
+        if (lane == 0) warp_sums[i][warp] = v;
+    }
+    asm volatile("barrier.cluster.wait;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            s[i] = __reduce_add_sync(0xffffffffu, lane < (int)(blockDim.x >> 5) ? warp_sums[i][lane] : 0);
+        if (lane == 0) {
+            uint32_t first;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(first) : "r"(smem_u32(&cta_sums[rank][0])));
+            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(first), "r"(s[0]), "r"(s[1]), "r"(s[2]),
+                         "r"(0)
+                         : "memory");
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+    if (rank != 0 || warp != 0) return;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s[i] = __reduce_add_sync(0xffffffffu, lane < (int)size ? cta_sums[lane & (kKuhnMaxCluster - 1)][i] : 0);
+    if (lane != 0) return;
+    if (!ok) atomicOr(a.err, ERRBIT_BAD_PAIR);
+    a.work[pair] = (unsigned long long)s[2];
+    finalize_pair(s[0], s[1], a.n_episodes, a.fin_out + 4 * (int64_t)pair);
+}
+
+// CTAs per pair of kuhn_cluster_kernel; 0: kuhn_eval_kernel takes the call. A pair's
+// cluster of at most 8 CTAs plays up to 4 hands a thread; longer calls are bound by
+// the generator and go over all the SMs.
+int kuhn_cluster(int32_t n_pairs, int64_t n_episodes, int n_sm) {
+    int c = kKuhnMaxCluster;
+    while (c > 1 && ((int64_t)n_pairs * c > 4 * (int64_t)n_sm || (int64_t)c * 64 > n_episodes)) c /= 2;
+    return n_episodes <= (int64_t)c * kKuhnMaxThreads * 4 ? c : 0;
 }
 
 // Exact expected seat-0 payoff: the 6 deals, each 1/6, times the betting tree.
@@ -131,8 +196,27 @@ __global__ void kuhn_exact_kernel(EvalArgs a, double* out) {
 
 }  // namespace
 
+bool kuhn_counts_itself(int32_t n_pairs, int64_t n_episodes, int n_sm) {
+    return kuhn_cluster(n_pairs, n_episodes, n_sm) != 0;
+}
+
 cudaError_t launch_kuhn_eval(const EvalArgs& a, int n_sm, cudaStream_t s) {
     if (a.n_pairs == 0) return cudaSuccess;
+    if (const int c = a.fin_out ? kuhn_cluster(a.n_pairs, a.n_episodes, n_sm) : 0) {
+        const int64_t per = (a.n_episodes + c - 1) / c;                      // hands of a CTA
+        const int64_t turns = (per + kKuhnMaxThreads - 1) / kKuhnMaxThreads;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)c;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(a.n_pairs * c));
+        cfg.blockDim = dim3((unsigned)(((per + turns - 1) / turns + 31) / 32 * 32));
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kuhn_cluster_kernel, a);
+    }
     int64_t blocks_per_pair = (a.n_episodes + 255) / 256;
     const int64_t cap = max(1, (n_sm * 8) / max(1, a.n_pairs));
     if (blocks_per_pair > cap) blocks_per_pair = cap;

@@ -55,6 +55,7 @@ struct malib_ctx {
     unsigned long long* acc = nullptr;
     int64_t acc_cap = 0;
     int64_t last_pairs = -1;           // n_pairs of the last Monte-Carlo evaluation
+    bool last_per_pair = false;        // its decisions are counted pair by pair
     int* d_err = nullptr;
     int32_t* d_pairs = nullptr;
     int64_t pairs_cap = 0;
@@ -652,7 +653,8 @@ int malib_eval_payoff_ex(malib_ctx* c, const int32_t* pair_ids, int32_t n_pairs,
         a.n_dec = c->acc + (int64_t)n_pairs * 2;
         a.work = c->acc + (int64_t)n_pairs * 2 + 1;
         c->last_pairs = n_pairs;
-        CK(launch_zero_u64(c->acc, (int64_t)n_pairs * 3 + 1, c->stream), "zero kernel");
+        c->last_per_pair = kind == MALIB_ENV_KUHN && kuhn_counts_itself(n_pairs, n_episodes, c->n_sm);
+        if (!c->last_per_pair) CK(launch_zero_u64(c->acc, (int64_t)n_pairs * 3 + 1, c->stream), "zero kernel");
         time_begin(c, &e0, &e1);
         if (kind == MALIB_ENV_KUHN) {
             a.fin_out = dout;                 // each pair's last block writes its row
@@ -676,7 +678,7 @@ int malib_eval_payoff_ex(malib_ctx* c, const int32_t* pair_ids, int32_t n_pairs,
         }
         time_end(c, e0, e1);
         if (!a.fin_out) CK(launch_finalize(c->acc, n_pairs, n_episodes, dout, c->stream), "finalize kernel");
-        c->launches += a.fin_out ? 2 : 3;
+        c->launches += c->last_per_pair ? 1 : a.fin_out ? 2 : 3;
     }
     if (host_out) {
         CK(cudaMemcpyAsync(payoff_out, dout, (size_t)n_pairs * 32, cudaMemcpyDeviceToHost,
@@ -980,11 +982,13 @@ int malib_eval_stats(malib_ctx* c, int64_t* n_decisions) {
     DeviceGuard g(c->device);
     *n_decisions = 0;
     if (c->last_pairs < 0) return fail(c, MALIB_ESTATE, "no Monte-Carlo evaluation has run");
-    unsigned long long v = 0;
-    CK(cudaMemcpyAsync(&v, c->acc + c->last_pairs * 2, 8, cudaMemcpyDeviceToHost, c->stream),
+    // [n_pairs][2] sums, the call's count, [n_pairs] counters
+    std::vector<unsigned long long> v(c->last_per_pair ? (size_t)c->last_pairs : 1);
+    CK(cudaMemcpyAsync(v.data(), c->acc + c->last_pairs * 2 + (c->last_per_pair ? 1 : 0), v.size() * 8,
+                       cudaMemcpyDeviceToHost, c->stream),
        "decision count");
     CK(cudaStreamSynchronize(c->stream), "sync");
-    *n_decisions = (int64_t)v;
+    for (unsigned long long d : v) *n_decisions += (int64_t)d;
     return MALIB_OK;
 }
 

@@ -101,6 +101,21 @@ def test_device_buffers_and_determinism(kuhn_ctx):
     np.testing.assert_array_equal(again, host)
 
 
+@pytest.mark.parametrize("n_pairs,n_eps", [(1, 1), (1, 127), (1, 128), (16, 24576), (16, 24577), (76, 6145), (77, 12288),
+                                           (77, 12289), (153, 6144), (305, 3072), (305, 3073)])
+def test_table_sums_on_both_sides_of_the_cluster_rule(kuhn_ctx, orc, n_pairs, n_eps):
+    """A cluster of 8, 4, 2 or 1 CTAs per pair up to 3,072 hands a CTA, blocks adding to global
+    accumulators past it: the integer sums and the decision count equal the oracle's."""
+    need_gpu()
+    ctx, w = kuhn_ctx
+    pairs = np.ascontiguousarray(np.resize(w.pair_ids, (n_pairs, 2)))
+    got = ctx.eval_payoff(pairs, n_eps, 21)
+    ref, tr = orc.kuhn_eval(tables(w), pairs, n_eps, 21, n_trace=n_eps)
+    np.testing.assert_array_equal(got[:, 2:], ref[:, 2:])
+    np.testing.assert_allclose(got[:, :2], ref[:, :2], rtol=1e-12, atol=1e-15)
+    assert ctx.eval_decisions() == int(tr[:, :, 2].sum())
+
+
 def test_invalid_arguments(kuhn_ctx):
     torch = need_gpu()
     ctx, w = kuhn_ctx
