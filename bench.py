@@ -28,7 +28,6 @@ sys.path.insert(0, ROOT)
 
 METRIC = "env-steps/sec incl. policy inference and payoff entries/sec on 1 GB300; % of roofline"
 UNIT = "env-steps/s"
-FP32_LANES_PER_SM = 128
 # DRAM bytes (read + write) per launch of each workload's dominant kernel, from
 # ncu (dram__bytes_read.sum + dram__bytes_write.sum). The fp32 rollout kernels were captured
 # on the benchmark's own workload with the two dram counters alone (one pass);
@@ -40,23 +39,38 @@ FP32_LANES_PER_SM = 128
 # not grow with the hands per pair; the learner's gradient kernel was captured
 # on the learner step's own workload.
 NCU_TRAFFIC_PER_LAUNCH = {
-    "leduc_eval_f32_t8_kernel": 1441536 + 512,
-    "kuhn_eval_kernel": 26880,
-    "spread_rollout_f32_kernel<3,18,64,0>": 1373184 + 2559883520,
+    "leduc_eval_x3_kernel<128>": 1298944 + 7424,
+    "kuhn_cluster_kernel": 20736,
+    "spread_rollout_x3_kernel<3,18,0>": 29975552 + 2587960064,
     "leduc_eval_tc_kernel": 19416064 + 490240,
-    "spread_rollout_f32_kernel<3,14,64,1>": 1683968 + 2068428800,
-    "spread_rollout_f32_kernel<2,11,64,2>": 1547520 + 1034004736,
+    "spread_rollout_x3_kernel<3,14,1>": 1442816 + 2073768960,
+    "spread_rollout_x3_kernel<2,11,2>": 3311616 + 1035926528,
     "spread_rollout_tc_kernel": (18220032 + 1910865664) * 2,
-    "learn_grad_kernel": 510880512 + 3277568,
-    "spread_rollout_f32_kernel<2,8,64,3>": 1031936 + 706821376,
-    "spread_rollout_f32_kernel<4,16,64,4>": 3663872 + 2780089856,
-    "spread_rollout_f32_kernel<2,14,64,6>": 2387712 + 1377357056,
+    "learn_grad_x3_kernel": 492022272 + 3917568,
+    "spread_rollout_x3_kernel<2,8,3>": 2444032 + 713326080,
+    "spread_rollout_x3_kernel<4,16,4>": 5594112 + 2782574592,
+    "spread_rollout_x3_kernel<2,14,6>": 3828224 + 1383427328,
 }
 
 
 def mlp_flop(dims):
     i, h1, h2, o = dims
     return 2 * (i * h1 + h1 * h2 + h2 * o)
+
+
+def tensor_peak(peaks, products):
+    """TFLOP/s of the tensor cores on products of the workload's type, and where the figure
+    comes from. A kernel is timed alone, launch by launch, with CUDA events, so the burst
+    figure of the measured cuBLAS bf16 GEMM is its peak; an fp32 product is six bf16 ones."""
+    if "bf16_tflops" in peaks:
+        peak = float(peaks["bf16_tflops"])
+        basis = "measured cuBLAS bf16 dense GEMM, burst (MEASURED_PEAKS.json bf16_tflops), of measured"
+    else:
+        peak = 1900.0
+        basis = "fallback bf16 dense burst 1.9 PFLOP/s (no MEASURED_PEAKS.json), of fallback"
+    if products > 1:
+        basis += f", over {products}: each fp32 product is {products} bf16 products on the tensor cores"
+    return peak / products, basis
 
 
 def parse():
@@ -471,7 +485,8 @@ def run_ours(args):
     else:
         d_out = torch.empty((w.n_pairs, 4), dtype=torch.float64, device=dev)
         flop_per_unit = mlp_flop(w.policies[0].dims) if w.env_kind == 2 else 0
-    tensor = args.workload in ("leduc_bf16", "spread8")
+    # an fp32 product is six bf16 products of the operands' three parts
+    products = 1 if args.workload in ("leduc_bf16", "spread8", "kuhn") else 6
 
     def step(seed):
         if rollout:
@@ -518,40 +533,27 @@ def run_ours(args):
     entries = sum_over_ranks(float(w.n_pairs * args.steps), world, dev) / (total_ms_max / 1e3)
 
     peaks = load_peaks()
-    sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak_tflops = n_sm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     achieved = (decisions * flop_per_unit / args.steps) / (kern_ms / kern_n / 1e3) / 1e12 \
         if kern_n else 0.0
-    kname = {"leduc": "leduc_eval_f32_t8_kernel", "kuhn": "kuhn_eval_kernel",
-             "spread3": "spread_rollout_f32_kernel<3,18,64,0>",
-             "adversary3": "spread_rollout_f32_kernel<3,14,64,1>",
-             "speaker_listener": "spread_rollout_f32_kernel<2,11,64,2>",
-             "push": "spread_rollout_f32_kernel<2,8,64,3>",
-             "tag": "spread_rollout_f32_kernel<4,16,64,4>",
-             "reference": "spread_rollout_f32_kernel<2,14,64,6>",
+    kname = {"leduc": "leduc_eval_x3_kernel<128>",
+             "kuhn": "kuhn_cluster_kernel" if w.n_episodes <= 24576 else "kuhn_eval_kernel",
+             "spread3": "spread_rollout_x3_kernel<3,18,0>",
+             "adversary3": "spread_rollout_x3_kernel<3,14,1>",
+             "speaker_listener": "spread_rollout_x3_kernel<2,11,2>",
+             "push": "spread_rollout_x3_kernel<2,8,3>",
+             "tag": "spread_rollout_x3_kernel<4,16,4>",
+             "reference": "spread_rollout_x3_kernel<2,14,6>",
              "leduc_bf16": "leduc_eval_tc_kernel",
              "spread8": "spread_rollout_tc_kernel"}[args.workload]
-    basis = (f"fp32 FMA: {n_sm} SMs (queried) x {FP32_LANES_PER_SM} lanes x 2 flop"
-             f" x {sm_max:.0f} MHz (max SM clock of MEASURED_PEAKS.json)")
-    if tensor:
-        # the kernel is timed alone, launch by launch, with CUDA events: the
-        # burst figure of the measured cuBLAS bf16 GEMM is its peak
-        if "bf16_tflops" in peaks:
-            peak_tflops = float(peaks["bf16_tflops"])
-            basis = "measured cuBLAS bf16 dense GEMM, burst (MEASURED_PEAKS.json bf16_tflops), of measured"
-        else:
-            peak_tflops = 1900.0
-            basis = "fallback bf16 dense burst 1.9 PFLOP/s (no MEASURED_PEAKS.json), of fallback"
-    roofline = {"bound": "tensor" if tensor else "alu", "achieved": achieved,
+    peak_tflops, basis = tensor_peak(peaks, products)
+    roofline = {"bound": "tensor", "achieved": achieved,
                 "peak": peak_tflops, "unit": "TFLOP/s",
                 "frac": achieved / peak_tflops if peak_tflops else None,
                 "traffic": NCU_TRAFFIC_PER_LAUNCH.get(kname),
                 "kernel": kname, "kernel_ms_per_launch": kern_ms / max(1, kern_n),
                 "peak_basis": basis,
                 "algorithmic": f"{flop_per_unit} flop per env-step (MLP forward, padding excluded)"}
-    if clk.get("sm_mhz") and not tensor:
-        roofline["frac_at_measured_clock"] = achieved / (peak_tflops * clk["sm_mhz"] / sm_max)
     if args.workload == "kuhn":
         # Kuhn's work is generator arithmetic: one Philox call per deal and one
         # per decision; the ceiling is the measured rate of a Philox-only kernel
@@ -583,7 +585,7 @@ def run_ours(args):
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": total_ms_max / args.steps,
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-                "dtype": "bf16" if tensor else "f32",
+                "dtype": "bf16" if args.workload in ("leduc_bf16", "spread8") else "f32",
                 "data": "synthetic", "config": config_of(w, args.workload),
                 "payoff_entries_per_s": entries if not rollout else None,
                 "env_steps_per_step": decisions / args.steps,
@@ -913,7 +915,7 @@ def run_learner(args):
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
           for _ in range(args.steps)]
     launches0 = ctx.launch_count()
-    ctx.set_timing(True)                 # learn_grad_kernel's own CUDA-event time
+    ctx.set_timing(True)                 # the gradient kernel's own CUDA-event time
     ctx.main_kernel_ms(reset=True)
     if world > 1:
         torch.distributed.barrier()
@@ -935,9 +937,7 @@ def run_learner(args):
     total_ms_max = max_over_ranks(total_ms, world, dev)
     value = sum_over_ranks(float(samples * args.steps), world, dev) / (total_ms_max / 1e3)
     peaks = load_peaks()
-    sm_max = float(peaks.get("sm_max_mhz", 2070.0))
-    n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    peak = n_sm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
+    peak, basis = tensor_peak(peaks, 6)
     grad_avg_ms = grad_ms / max(grad_n, 1)
     achieved = samples * learn_flop(dims) / (grad_avg_ms / 1e3) / 1e12
     e2e = None
@@ -1001,12 +1001,11 @@ def run_learner(args):
                                        f"{w.n_episodes}episodes_pop{n_pol}", "samples_per_step": samples,
                            "policies": n_pol,
                            "l2": "flushed (256 MiB write) before every timed step"},
-                "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                              "frac": achieved / peak,
-                             "traffic": None if ppo else NCU_TRAFFIC_PER_LAUNCH.get("learn_grad_kernel"),
-                             "kernel": "learn_grad_kernel",
-                             "peak_basis": f"fp32 FMA: {n_sm} SMs (queried) x {FP32_LANES_PER_SM} lanes x 2 "
-                                           f"flop x {sm_max:.0f} MHz",
+                             "traffic": None if ppo else NCU_TRAFFIC_PER_LAUNCH.get("learn_grad_x3_kernel"),
+                             "kernel": "learn_grad_x3_kernel",
+                             "peak_basis": basis,
                              "algorithmic": f"{learn_flop(dims)} flop per sample (forward and backward, "
                                             f"bias sums excluded) x {samples} samples per launch",
                              "kernel_ms": grad_avg_ms, "step_share": grad_avg_ms / (total_ms / args.steps)},

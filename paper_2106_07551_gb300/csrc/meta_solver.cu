@@ -3,10 +3,11 @@
 // payoffs aggregated under the equilibrium). A[i][j] is seat 0's payoff when
 // row policy i meets column policy j; the games are zero-sum.
 //
-// One CTA solves one game (batched over a grid of games). Everything a game
-// needs stays on chip: the payoff matrix (or the LP tableau) in shared memory
-// when it fits, cumulative payoffs in registers, and each iteration's argmax /
-// argmin in warp shuffles plus one cross-warp step.
+// One CTA solves one game of fictitious play, the sides on different warps and
+// each play's argmax / argmin by integer warp reductions; an LP is dealt over the
+// CTAs of a cluster by columns. What a game needs stays on chip where it fits: the
+// payoff matrix (or the LP tableau) in shared memory, cumulative payoffs in
+// registers.
 #include <cstdint>
 #include <type_traits>
 
