@@ -63,7 +63,7 @@ typedef enum malib_policy_kind {
 } malib_policy_kind;
 
 typedef enum malib_dtype {
-    MALIB_F32 = 0,            /* fp32 weights, fp32 FMA forward */
+    MALIB_F32 = 0,            /* fp32 weights, fp32 forward */
     MALIB_BF16 = 1            /* bf16 weights and layer inputs, fp32 accumulation */
 } malib_dtype;
 
