@@ -310,7 +310,7 @@ int malib_eval_payoff_ex(malib_ctx* ctx, const int32_t* pair_ids, int32_t n_pair
  *    malib_eval_stats does not report its decision count.
  *  - The first call on a device looks the array's device address up
  *    (cudaGetSymbolAddress); make that first call before any stream capture.
- *  - Every call shares the array and clears it first; calls that overlap on
+ *  - Every call shares the array and clears what it adds to; calls that overlap on
  *    the GPU (other streams or contexts on the same device) race on it.
  */
 int malib_eval_payoff_noalloc(malib_ctx* ctx, const int32_t* pair_ids, int32_t n_pairs,
