@@ -274,8 +274,13 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
 }
+// Without .aligned: a warp's lanes may arrive one by one (its loops before the
+// barrier have lane-dependent trip counts).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 struct LpShape {
@@ -304,6 +309,8 @@ __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
     __shared__ int basis[kLpMaxDim], label[kLpMaxDim];       // label: variable of each own column
     __shared__ Cand red[2][kLpWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if constexpr (kCluster) cluster_arrive();                // this CTA runs: its peers may store into it
+    bool peers_run = false;
     const int m = sh.m, n = sh.n, hs = sh.hs;
     const int rank = kCluster ? (int)cluster_rank() : 0, size = kCluster ? sh.cluster : 1;
     const int c_lo = rank * sh.cols, w = max(0, min(sh.cols, n - c_lo));   // own columns
@@ -338,6 +345,11 @@ __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
         for (int r = tid; r < m; r += kLpThreads) basis[r] = n + r;
         for (int c = tid; c < w; c += kLpThreads) label[c] = c_lo + c;
         __syncthreads();
+        if constexpr (kCluster) {
+            // before the first remote access (a CTA that has not started has no shared memory yet)
+            if (!peers_run) cluster_wait();
+            peers_run = true;
+        }
 
         const int max_pivots = pivot_limit > 0 ? pivot_limit : 50 * (m + n) + 1000;
         bool done = false, bland = false;

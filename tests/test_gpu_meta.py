@@ -123,17 +123,36 @@ def test_lp_value_and_equilibrium(ctx, m, n):
     check_lp(tables, *run_lp(ctx, tables))
 
 
-@pytest.mark.parametrize("G,m,n", [(1, 40, 40), (1, 39, 41), (4, 100, 17), (20, 45, 83), (50, 64, 33), (3, 33, 130),
-                                   (2, 512, 9), (1, 300, 290), (40, 300, 200), (70, 200, 150)])
-def test_lp_games_over_clusters(ctx, G, m, n):
+@pytest.mark.parametrize("G,m,n,whole", [(1, 40, 40, 0), (1, 40, 40, 1), (1, 39, 41, 0), (1, 39, 41, 1), (4, 100, 17, 1),
+                                         (20, 45, 83, 1), (50, 64, 33, 1), (3, 33, 130, 1), (2, 512, 9, 1),
+                                         (1, 300, 290, 0), (1, 300, 290, 1), (40, 300, 200, 1), (70, 200, 150, 1)])
+def test_lp_games_over_clusters(ctx, G, m, n, whole):
     """Columns dealt over 8, 4, 2 and 1 CTAs, CTAs with fewer columns or none,
-    tableaus on and off chip; integer tables in the last third tie often."""
+    tableaus on and off chip; the last `whole` tables hold small integers, which tie
+    often, the others normal deviates."""
     rng = np.random.default_rng(m * n + G)
     tables = rng.normal(size=(G, m, n))
-    tables[-1] = rng.integers(-2, 3, size=(m, n))
+    if whole:
+        tables[-1] = rng.integers(-2, 3, size=(m, n))
     gx, gy, gv = run_lp(ctx, tables)
     some = sorted({0, G // 2, G - 1})
     check_lp(tables[some], gx[some], gy[some], gv[some])
+
+
+def test_lp_clusters_back_to_back(ctx):
+    """One game on a cluster of eight CTAs, launched 40 times in a row: every launch
+    starts its clusters anew and gives the same bits."""
+    torch = need_gpu()
+    rng = np.random.default_rng(5)
+    tables = rng.normal(size=(1, 64, 64))
+    P = torch.from_numpy(tables).cuda()
+    x, y = (torch.zeros((40, 1, 64), dtype=torch.float64, device="cuda") for _ in range(2))
+    v = torch.zeros((40, 1), dtype=torch.float64, device="cuda")
+    for i in range(40):
+        ctx.meta_lp_nash(P, x[i], y[i], v[i])
+    ctx.sync()
+    check_lp(tables, x[0].cpu().numpy(), y[0].cpu().numpy(), v[0].cpu().numpy())
+    assert torch.equal(x, x[:1].expand_as(x)) and torch.equal(y, y[:1].expand_as(y)) and torch.equal(v, v[:1].expand_as(v))
 
 
 def test_lp_closed_forms_and_degenerate(ctx):

@@ -28,3 +28,28 @@ def test_min_of_rounded_roots_is_root_of_min():
     rng = np.random.default_rng(0)
     x = (rng.random((200_000, 8)) * 8).astype(np.float32)
     np.testing.assert_array_equal(np.sqrt(x).min(axis=1), np.sqrt(x.min(axis=1)))
+
+
+def test_remote_shared_memory_waits_for_its_cta():
+    """A CTA's shared memory may be accessed by its cluster's other CTAs only once it
+    runs: every kernel that stores to or loads from a peer arrives at and waits for a
+    cluster barrier first. The barriers follow code in which lanes diverge, so none
+    is the .aligned form."""
+    csrc = os.path.join(ROOT, "paper_2106_07551_gb300", "csrc")
+    kernels = 0
+    for name in sorted(os.listdir(csrc)):
+        src = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        assert not re.search(r"barrier\.cluster\.[a-z.]*aligned", src), name
+        # one-line helpers that arrive or wait, by name
+        call = {w: [f"barrier.cluster.{w}"] + [f + "()" for f in
+                re.findall(r"void (\w+)\(\) \{ asm volatile\(\"barrier\.cluster\." + w, src)] for w in ("arrive", "wait")}
+        for body in re.split(r"(?=__global__)", src)[1:]:
+            remote = re.search(r"(?:st|ld)\.shared::cluster", body)
+            if not remote:
+                continue
+            kernels += 1
+            before = body[:remote.start()]
+            arrive = min((before.find(c) for c in call["arrive"] if c in before), default=-1)
+            assert arrive >= 0, f"{name}: no cluster barrier before the first remote access"
+            assert any(c in before[arrive:] for c in call["wait"]), f"{name}: no wait before the first remote access"
+    assert kernels == 2                  # Kuhn's clusters and the linear program's
