@@ -172,6 +172,20 @@ def test_lp_closed_forms_and_degenerate(ctx):
     assert abs(gv[2] - 0.25) < 1e-15
 
 
+@pytest.mark.parametrize("table,x,y", [
+    ([[-3, -1, 2], [3, -1, 2], [3, 1, -2]], [0, 1 / 2, 1 / 2], [0, 2 / 3, 1 / 3]),
+    ([[3, 1, 2, -3], [3, -3, -1, 1], [-2, 0, 2, -2], [-3, -3, -1, 1]], [1 / 2, 1 / 2, 0, 0], [0, 1 / 2, 0, 1 / 2]),
+    ([[2, 3, 0], [2, -2, -3], [-1, -3, 1], [-3, -2, -2], [-2, 3, 0]], [4 / 7, 0, 3 / 7, 0, 0], [0, 1 / 7, 6 / 7]),
+    ([[3, 3, 3, 3, 1, -3], [-2, 3, -3, 3, -3, -3], [0, -1, 2, -2, 2, 2], [2, 0, 1, 0, -3, -2], [-2, 0, 2, -1, -2, 0]],
+     [2 / 5, 0, 3 / 5, 0, 0], [0, 0, 0, 1 / 2, 0, 1 / 2])])
+def test_lp_equal_ratios_tie(ctx, table, x, y):
+    """Rows whose ratios are equal rationals tie, and the lowest basic variable leaves:
+    the equilibrium is the one that the same rules reach in exact rational arithmetic
+    (these games have others)."""
+    gx, gy, _ = run_lp(ctx, np.array([table], float))
+    assert np.abs(gx[0] - x).max() < 1e-12 and np.abs(gy[0] - y).max() < 1e-12, (gx, gy)
+
+
 def test_lp_off_chip(ctx):
     rng = np.random.default_rng(77)
     tables = rng.normal(size=(2, 300, 200))          # tableau 301 x 501 fp64 > 200 KB
