@@ -226,6 +226,18 @@ struct CtxView {
     bool tc_layout;               // bf16 tensor-core images in the arena (else fp32 layouts)
 };
 bool ctx_view(const void* ctx, CtxView* v);
+// Selects a device and, when it goes, the one selected before.
+struct DevSel {
+    int prev = -1;
+    bool ok = true;
+    explicit DevSel(int dev) {
+        if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
+        ok = cudaSetDevice(dev) == cudaSuccess;
+    }
+    ~DevSel() {
+        if (prev >= 0) cudaSetDevice(prev);
+    }
+};
 // Where a pointer lives, by cudaPointerGetAttributes: host memory (pageable,
 // pinned or unknown), device memory of `device` (or managed memory), or device
 // memory of another GPU, which no kernel of a context on `device` may touch.

@@ -562,18 +562,6 @@ namespace {
 // Device memory of the context's own device.
 bool dev_ptr(int device, const void* p) { return p && ptr_where(p, device) == kPtrHere; }
 
-struct DevSel {
-    int prev = -1;
-    bool ok = true;
-    explicit DevSel(int dev) {
-        if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        ok = cudaSetDevice(dev) == cudaSuccess;
-    }
-    ~DevSel() {
-        if (prev >= 0) cudaSetDevice(prev);
-    }
-};
-
 int check_table(malib_ctx* ctx, int device, const double* payoff, int32_t G, int32_t m, int32_t n,
                 int32_t stride, int32_t max_dim) {
     if (G < 0) return ctx_fail(ctx, MALIB_EINVAL, "n_games < 0");
