@@ -30,6 +30,19 @@ __device__ __forceinline__ unsigned long long f2_relu(unsigned long long v) {
     return r;
 }
 
+// max(v, 0) that keeps a NaN (fmaxf(NaN, 0) is 0).
+__device__ __forceinline__ float relu_nan(float v) {
+    float r;
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_relu_nan(unsigned long long v) {
+    const float2 q = f2_split(v);
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(relu_nan(q.x)), "f"(relu_nan(q.y)));
+    return r;
+}
+
 __device__ __forceinline__ unsigned long long f2_pack(uint32_t lo, uint32_t hi) {
     unsigned long long r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));

@@ -31,6 +31,14 @@
 // images, [wl 0 0], [wm wm 0] and [wh wh wh], each multiplied with the steps of
 // X that it reaches (2 + 3 + 4 steps for 18 inputs, where parts padded one by
 // one would take 12); the steps of the last image run from l to h.
+//
+// An infinity, and a finite value that rounds to a bf16 infinity (from 3.3962e38),
+// has no such parts: they are infinite and NaN, and so are the products. The ReLUs
+// keep a NaN, which makes every unit of the next layer and every logit NaN, so the
+// first logit tells, and the caller takes that row again in fp32 FMAs
+// (forward_fma), which give such weights and activations their IEEE meaning. At
+// the other end, values below 2^-110 lose their low parts to bf16's smallest
+// magnitude, 2^-133: that shows in a sum only next to weights beyond 2^100.
 #pragma once
 
 #include <cstdint>
@@ -48,6 +56,35 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t& h, uint32_t
     const float r1 = __fsub_rn(v1, __uint_as_float(h & 0xffff0000u));
     m = tc::pack_bf16(r0, r1);
     l = tc::pack_bf16(__fsub_rn(r0, __uint_as_float(m << 16)), __fsub_rn(r1, __uint_as_float(m & 0xffff0000u)));
+}
+
+// True for a row whose parts were not finite somewhere (any of its logits tells).
+__device__ __forceinline__ bool parts_failed(float logit) { return !(fabsf(logit) <= 3.402823466e38f); }
+
+// The forward of one row x by one thread in fp32 FMAs (bias first, inputs
+// ascending), from the population's image; slow, for rows whose parts failed.
+template <int IN, int H, int A>
+__device__ __noinline__ void forward_fma(const float* __restrict__ img, const float* x, float* lg) {
+    using L = F32Layout<IN, H, A>;
+    float h1[H], s[A];
+#pragma unroll 1
+    for (int j = 0; j < H; ++j) {
+        float z = __ldg(img + L::kB1 + j);
+        for (int k = 0; k < IN; ++k) z = fmaf(x[k], __ldg(img + L::kW1T + k * H + j), z);
+        h1[j] = fmaxf(z, 0.f);
+    }
+    for (int a = 0; a < A; ++a) s[a] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < H; ++j) {
+        float z = __ldg(img + L::kB2 + j);
+#pragma unroll 8
+        for (int k = 0; k < H; ++k) z = fmaf(h1[k], __ldg(img + L::kW2T + k * H + j), z);
+        z = fmaxf(z, 0.f);
+#pragma unroll
+        for (int a = 0; a < A; ++a) s[a] = fmaf(z, __ldg(img + L::kW3 + a * H + j), s[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < A; ++a) lg[a] = s[a] + __ldg(img + L::kB3 + a);
 }
 
 template <int IN, int A>
@@ -209,8 +246,8 @@ struct MlpX3 {
             tc::tmem_ld32x1(tbase + lane_q + kD1 + 32u * c, v);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-                split3(fmaxf(__uint_as_float(v[2 * i]), 0.f), fmaxf(__uint_as_float(v[2 * i + 1]), 0.f), w[0][i],
-                       w[1][i], w[2][i]);
+                split3(relu_nan(__uint_as_float(v[2 * i])), relu_nan(__uint_as_float(v[2 * i + 1])), w[0][i], w[1][i],
+                       w[2][i]);
 #pragma unroll
             for (int q = 0; q < 3; ++q) tc::tmem_st16(tbase + lane_q + h_col(q, 2 * c), w[q]);
         }
@@ -234,7 +271,7 @@ struct MlpX3 {
             tc::tmem_ld32x1(tbase + lane_q + kD2 + 32u * c, d);
             u64 z[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) z[i] = f2_relu(f2_pack(d[2 * i], d[2 * i + 1]));
+            for (int i = 0; i < 16; ++i) z[i] = f2_relu_nan(f2_pack(d[2 * i], d[2 * i + 1]));
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
 #pragma unroll

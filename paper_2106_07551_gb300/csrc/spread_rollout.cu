@@ -325,6 +325,13 @@ __global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
                     if (busy) {
                         float lg[A];
                         M::logits(tb, lane_q, pol, lg);
+                        if (mine && parts_failed(lg[0])) {
+                            // (its observation is in the trajectory since before layer 2)
+                            float z[A];
+                            forward_fma<IN, M::H, A>(a.arena + a.pol_offset[a.pairs[pair * N + i]], a.obs + (ix + i) * XS, z);
+#pragma unroll
+                            for (int k = 0; k < A; ++k) lg[k] = z[k];
+                        }
                         if (mine) {
                             const unsigned legal = (kScen == kSpeakerListener && i == 0) ? kSlSpeakerLegal : (1u << A) - 1u;
                             act_pk |= (uint32_t)sample_masked<A>(lg, legal, uu) << (4 * i);

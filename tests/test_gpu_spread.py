@@ -8,7 +8,8 @@ import numpy as np
 import pytest
 
 import workloads
-from gpu_util import context, load_population, logits_close, need_gpu, spec_of
+from gpu_util import (context, load_population, logits_close, logits_same_class, need_gpu, plant_odd_weights,
+                      spec_of)
 
 pytestmark = pytest.mark.gpu
 
@@ -71,6 +72,30 @@ def test_units_over_groups_and_items(orc, n_envs, epp, n_eps):
     for lo in (0, n_envs // 2, n_envs - 9):
         check(orc, w, g, n_eps, 99, lo, lo + 9)
     ctx.close()
+
+
+@pytest.mark.parametrize("make,kw,n_eps", [(workloads.spread, {"n_agents": 3}, 3), (workloads.tag, {}, 2),
+                                           (workloads.reference, {}, 1)])
+def test_non_finite_and_huge_weights(orc, make, kw, n_eps):
+    """Infinite, NaN and huge weights (a diverged policy's) show in the logits as IEEE
+    arithmetic has them: the recorded logits of every agent's own observations. The
+    agents of a row with such a policy do not disturb the others' rows."""
+    need_gpu()
+    w = make(n_envs=12 * 40, pop=16, envs_per_pair=40, with_bias=True, seed=21, **kw)
+    plant_odd_weights(w.policies)
+    ctx = context()
+    load_population(ctx, w)
+    g = rollout(ctx, w, n_eps, 77)
+    ctx.close()
+    combo = np.asarray(w.pair_ids).repeat(40, axis=0)               # [env][agent] -> policy
+    for p, pol in enumerate(w.policies):
+        env, agent = np.nonzero(combo == p)
+        x = g["obs"][:, :, env, agent, :w.obs_dim].reshape(-1, w.obs_dim)
+        ref = orc.mlp_forward(pol.params, pol.dims, x)
+        # a huge weight times a speed above 1 (tag) overflows fp32, but not the oracle's 64 bits
+        in_range = np.abs(x[:, 0]) <= 1.0 if p % 8 == 3 else slice(None)
+        logits_same_class(g["logits"][:, :, env, agent].reshape(ref.shape)[in_range], ref[in_range], pol.params, pol.dims,
+                          x[in_range])
 
 
 @pytest.mark.parametrize("rho", [0.0, 0.3, 1.0])
