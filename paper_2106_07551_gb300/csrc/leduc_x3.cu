@@ -217,8 +217,8 @@ struct LeducX3 {
             tc::tmem_ld32x1(tb + lane_q + d1_col(b), v);
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-                split3(fmaxf(__uint_as_float(v[2 * i]), 0.f), fmaxf(__uint_as_float(v[2 * i + 1]), 0.f), w[0][i],
-                       w[1][i], w[2][i]);
+                split3(relu_nan(__uint_as_float(v[2 * i])), relu_nan(__uint_as_float(v[2 * i + 1])), w[0][i], w[1][i],
+                       w[2][i]);
 #pragma unroll
             for (int q = 0; q < 3; ++q) tc::tmem_st16(tb + lane_q + hid_col(b, q), w[q]);
         }
@@ -233,8 +233,8 @@ struct LeducX3 {
         tc::tmem_ld32x1(tb + lane_q + kD2 + 32u * hh, d);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const unsigned long long z0 = f2_relu(f2_pack(d[4 * i], d[4 * i + 1]));
-            const unsigned long long z1 = f2_relu(f2_pack(d[4 * i + 2], d[4 * i + 3]));
+            const unsigned long long z0 = f2_relu_nan(f2_pack(d[4 * i], d[4 * i + 1]));
+            const unsigned long long z1 = f2_relu_nan(f2_pack(d[4 * i + 2], d[4 * i + 3]));
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(f + q * H + 4 * i);
@@ -456,6 +456,12 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                         LeducHand h;
                         int t;
                         unpack_hand(w, h, t);
+                        if (parts_failed(lg[0])) {
+                            float ob[17], z[3];
+                            leduc_obs(h, ob);
+                            forward_fma<17, H, 3>(a.arena + a.pol_offset[pol], ob, z);
+                            lg[0] = z[0]; lg[1] = z[1]; lg[2] = z[2];
+                        }
                         const int act = sample_masked<3>(lg, leduc_legal(h), u);
                         const int64_t e = e_lo + id;
                         const bool rec = kDump && e < a.n_dump;

@@ -12,7 +12,8 @@ import numpy as np
 import pytest
 
 import workloads
-from gpu_util import context, four_se_rule, load_population, logits_close, need_gpu
+from gpu_util import (context, four_se_rule, load_population, logits_close, logits_same_class, need_gpu,
+                      plant_odd_weights)
 
 pytestmark = pytest.mark.gpu
 
@@ -111,6 +112,29 @@ def test_tile_edges(orc, hidden, n_eps):
     w.pair_ids = pairs
     check_replay(orc, w, res, {k: v.cpu().numpy() for k, v in dump.items()}, n_eps, 17, n_eps, full=True)
     ctx.close()
+
+
+@pytest.mark.parametrize("hidden,n_eps", [(64, 300), (128, 300)])
+def test_non_finite_and_huge_weights(orc, hidden, n_eps):
+    """Infinite, NaN and huge weights (a diverged policy's) show in the logits as IEEE
+    arithmetic has them, and other policies' hands are not disturbed."""
+    need_gpu()
+    w = workloads.leduc(pop=8, hidden=hidden, with_bias=True, seed=hidden + 3)
+    plant_odd_weights(w.policies)
+    ctx = context()
+    load_population(ctx, w)
+    _, d = run_dumped(ctx, w, n_eps, 55, n_eps)
+    ctx.close()
+    acted = d["action"] != 255
+    # the acting seat is not recorded: replayed with the recorded actions' logits
+    _, rec = orc.leduc_eval([p.params for p in w.policies], w.policies[0].dims, w.pair_ids, n_eps, 55, n_rec=n_eps,
+                            ext_logits=np.where(np.arange(3) == d["action"][..., None], 80.0, 0.0).astype(np.float32))
+    np.testing.assert_array_equal(rec["obs"][acted], d["obs"][..., :17][acted])
+    actor = w.pair_ids[np.arange(w.n_pairs)[:, None, None], rec["seat"].clip(0)]
+    for p, pol in enumerate(w.policies):
+        mine = acted & (actor == p)
+        x = d["obs"][..., :17][mine]
+        logits_same_class(d["logits"][mine], orc.mlp_forward(pol.params, pol.dims, x), pol.params, pol.dims, x)
 
 
 @pytest.mark.parametrize("action", [1, 2])
