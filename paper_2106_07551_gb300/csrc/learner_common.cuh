@@ -6,6 +6,9 @@
 
 namespace malib {
 
+constexpr int kH = 64, kA = 5;                           // hidden width, actions
+constexpr int kTile = 128, kThreads = 256;               // samples of a tile, threads of a CTA
+
 // Sample s of the policy's sample order: (slot, episode, step, env) -> the
 // trajectory index of its (episode, step, env, agent).
 __device__ __forceinline__ int64_t sample_index(const LearnArgs& a, const int32_t* slots, int64_t s, int epp) {

@@ -35,14 +35,12 @@
 // (learn_grad_kernel 2.2e-7 .. 3.3e-7).
 #include "device_common.cuh"
 #include "f32x2.cuh"
-#include "learner_common.cuh"
+#include "learner_fma.cuh"
 #include "mlp_x3.cuh"
 
 namespace malib {
 
 namespace {
-
-constexpr int kH = 64, kA = 5, kTile = 128, kThreads = 256;
 
 template <int PP>                          // input width rounded up (zeros past the width)
 struct LearnX3 {
@@ -298,6 +296,15 @@ __device__ __noinline__ uint32_t chain_signs(const float* __restrict__ pol, int 
     return out;
 }
 
+// Tiles once more in fp32 FMAs, from the CTA's first policy whose partial is not
+// finite to its last one: an infinity, a NaN or a value beyond bf16's range
+// (3.3962e38) among the weights, the activations, the observations or the gradients
+// has no parts (mlp_x3.cuh), and what comes out then shows it (the ReLUs keep a NaN,
+// which reaches the row's logits and with them db3) but need not be what IEEE
+// arithmetic gives. Called at the kernel's end, where nothing is live: from flush
+// it cost the tiles 1 to 2 %.
+__device__ __noinline__ void redo_tiles(LearnArgs a, float* sm, int64_t lo, int64_t hi) { learn_tiles_fma(a, sm, lo, hi); }
+
 template <int PP>
 __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a) {
     using E = LearnX3<PP>;
@@ -308,6 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
     __shared__ __align__(8) uint64_t bars[4];
     __shared__ uint32_t tmem_base, dead;
     __shared__ int step[4];                              // 128 samples as (env, step, episode, slot)
+    __shared__ int64_t redo[2];                          // tiles for redo_tiles (none: empty)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int qt = warp & 3, hh = warp >> 2, r = 32 * qt + lane;      // lane quarter, half, row
     const int in = a.in;
@@ -318,6 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
     if (tid == 0) {
         for (int i = 0; i < 4; ++i) mbar_init(&bars[i], 1);
         dead = 0u;
+        redo[0] = redo[1] = 0;
         int q = kTile / epp;
         step[0] = kTile - q * epp;
         step[1] = q % a.T;
@@ -370,14 +379,19 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
     constexpr int kChunks = E::kK1 / 16;                 // 16-column chunks of X's block; this thread's: hh, hh + 2
     auto flush = [&] {
         float* out = a.gpart + ((int64_t)b * a.grid + blockIdx.x) * (P + 2);
+        bool finite = true;
+        auto put = [&](int e, float v) {
+            out[e] = v;
+            finite = finite && fabsf(v) <= 3.402823466e38f;
+        };
         const int oW2 = kH * in + kH, oW3 = oW2 + kH * kH + kH;
         float* S = reinterpret_cast<float*>(sm + E::kH1);            // [64][kK1] of d1^T X
         float* R = reinterpret_cast<float*>(sm + E::kDU);            // [7][128]
         float* R3 = R + 7 * 128;                                      // [8][5][64]
         if (qt < 2) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) out[oW2 + r * kH + 32 * hh + i] = gacc[i];
-            if (hh == 0) out[oW2 + kH * kH + r] = gb2;
+            for (int i = 0; i < 32; ++i) put(oW2 + r * kH + 32 * hh + i, gacc[i]);
+            if (hh == 0) put(oW2 + kH * kH + r, gb2);
         } else {
 #pragma unroll
             for (int c = 0; c < (kChunks + 1) / 2; ++c)
@@ -397,22 +411,25 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
         for (int e = tid; e < kH * in; e += kThreads) {
             const int j = e / in, f = e - j * in;
             const float* s = S + j * E::kK1;
-            out[e] = (s[2 * PP + f] + s[PP + f]) + s[f];
+            put(e, (s[2 * PP + f] + s[PP + f]) + s[f]);
         }
-        if (tid < kH) out[kH * in + tid] = S[tid * E::kK1 + E::kOnes];
+        if (tid < kH) put(kH * in + tid, S[tid * E::kK1 + E::kOnes]);
         for (int e = tid; e < kA * kH; e += kThreads) {
             float v[8];
 #pragma unroll
             for (int g = 0; g < 8; ++g) v[g] = R3[g * kA * kH + e];
-            out[oW3 + e] = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+            put(oW3 + e, ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
         }
         if (warp < 7) {
             float s = (R[warp * 128 + lane] + R[warp * 128 + 32 + lane]) + (R[warp * 128 + 64 + lane] + R[warp * 128 + 96 + lane]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) out[warp < 5 ? oW3 + kA * kH + warp : P + warp - 5] = s;
+            if (lane == 0) put(warp < 5 ? oW3 + kA * kH + warp : P + warp - 5, s);
         }
-        __syncthreads();
+        if (__syncthreads_or(!finite) && tid == 0) {
+            redo[0] = redo[1] > redo[0] ? redo[0] : max(lo, a.tile_off[b]);
+            redo[1] = min(hi, a.tile_off[b + 1]);
+        }
     };
     // this row's sample of a tile of policy b (both threads the action, return and
     // behavior logits; the first the observation): the loads only
@@ -573,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
                 m1 |= v[i] > 0.f ? 1u << i : 0u;
-                v[i] = fmaxf(v[i], 0.f);
+                v[i] = relu_nan(v[i]);
             }
             E::spread(v, tq, hh, true, sm + E::kH1 + (odd ? 2 * E::kPartH1 : 0u),
                       odd ? -(int)E::kPartH1 : (int)E::kPartH1, r, 32 * hh);
@@ -593,7 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
             for (int i = 0; i < 32; ++i) h2[i] = __uint_as_float(d[i]);
             settle(h2, 2, odd);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) h2[i] = fmaxf(h2[i], 0.f);
+            for (int i = 0; i < 32; ++i) h2[i] = relu_nan(h2[i]);
             float4* p = reinterpret_cast<float4*>(sm + E::h2_at(r)) + 8 * hh;
 #pragma unroll
             for (int i = 0; i < 8; ++i) p[i] = make_float4(h2[4 * i], h2[4 * i + 1], h2[4 * i + 2], h2[4 * i + 3]);
@@ -767,14 +784,17 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
     tc::fence_before_sync();
     flush();
     if (warp == 0) tc::tmem_dealloc(tmem_base, 512);
+    __syncthreads();
+    if (redo[1] > redo[0]) redo_tiles(a, reinterpret_cast<float*>(sm), redo[0], redo[1]);
 }
 
 template <int PP>
 cudaError_t launch_pp(const LearnArgs& a, cudaStream_t s) {
+    constexpr size_t bytes = LearnX3<PP>::kBytes > kSBytes ? LearnX3<PP>::kBytes : kSBytes;    // redo_tiles needs kSBytes
     const cudaError_t e = cudaFuncSetAttribute(learn_grad_x3_kernel<PP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)LearnX3<PP>::kBytes);
+                                               (int)bytes);
     if (e != cudaSuccess) return e;
-    learn_grad_x3_kernel<PP><<<a.grid, kThreads, LearnX3<PP>::kBytes, s>>>(a);
+    learn_grad_x3_kernel<PP><<<a.grid, kThreads, bytes, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -17,7 +17,7 @@ import pytest
 import oracle
 import workloads
 from oracle import learner
-from gpu_util import context, load_population, logits_close, need_gpu, spec_of
+from gpu_util import context, load_population, logits_close, need_gpu, plant_odd_weights, spec_of
 
 pytestmark = pytest.mark.gpu
 
@@ -449,3 +449,50 @@ def test_relu_inputs_within_rounding_of_zero(in_dim):
     got = g[:64 * in_dim].reshape(64, in_dim)[tiny]
     np.testing.assert_allclose(got, want, rtol=0, atol=1e-4 * np.abs(want).max())
     ctx.close()
+
+
+@pytest.mark.parametrize("in_dim", [10, 16, 18])
+@pytest.mark.parametrize("where", list(range(7)) + ["observations", "rewards"])
+def test_non_finite_and_huge_values(in_dim, where):
+    """Infinite, NaN and huge weights (kinds 0 .. 6), observations and rewards: the gradient
+    and the statistics have the NaN and infinities, and otherwise the values, that the
+    general kernel gives for the same samples (24 wide: zero features with zero weights
+    behind the others). Policy 1, whose samples lie among policy 0's, keeps its values."""
+    torch = need_gpu()
+    w, tr, traj = synthetic(in_dim, 128, seed=6)
+    if where == "observations":
+        tr["obs"][0, 2, 5, 0, 3], tr["obs"][1, 3, 7, 1, 4], tr["obs"][2, 0, 9, 0, 0] = np.inf, 3.4e38, np.nan
+    elif where == "rewards":
+        tr["reward"][1, 4, 11, 0], tr["reward"][2, 6, 300, 1] = -np.inf, 3.4e38
+    else:
+        plant_odd_weights([w.policies[1]] * where + [w.policies[0]])
+        w.policies[1].params = workloads.random_mlp(np.random.default_rng(1), w.policies[1].dims, True)
+    wide = workloads.spread(n_agents=2, n_envs=w.n_envs, pop=2, obs_dim=24, episode_len=7, envs_per_pair=128, seed=1)
+    wide.pair_ids = w.pair_ids
+    for p, q in zip(w.policies, wide.policies):
+        W1 = np.zeros((64, 24), np.float32)
+        W1[:, :in_dim] = p.params[:64 * in_dim].reshape(64, in_dim)
+        q.params = np.concatenate([W1.ravel(), p.params[64 * in_dim:]])
+    obs = np.zeros(tr["obs"].shape[:-1] + (24,), np.float32)
+    obs[..., :in_dim] = tr["obs"][..., :in_dim]
+    out = []
+    for v, o in ((w, tr["obs"]), (wide, obs)):
+        ctx = context()
+        load_population(ctx, v)
+        t = {"obs": torch.from_numpy(o).cuda(), "action": traj["action"], "reward": torch.from_numpy(tr["reward"]).cuda()}
+        P = int(blocks(v.policies[0].dims)[-1])
+        g, st = torch.zeros((2, P), device="cuda"), torch.zeros((2, 4), dtype=torch.float64, device="cuda")
+        ctx.learn_pg_batch(spec_of(v), v.pair_ids, 3, t, [0, 1], 0.9, 0.01, g, st)
+        ctx.close()
+        g, d = g.cpu().numpy(), v.policies[0].dims[0]
+        out.append((np.concatenate([g[:, :64 * d].reshape(2, 64, d)[..., :in_dim].reshape(2, -1), g[:, 64 * d:]], 1),
+                    st.cpu().numpy()))
+    (g, st), (want, want_st) = out
+    np.testing.assert_allclose(st, want_st, rtol=1e-5, atol=1e-6)        # (equal NaN and infinities)
+    dims = w.policies[0].dims
+    for pid in (0, 1):
+        np.testing.assert_array_equal(np.where(np.isfinite(g[pid]), 0, g[pid]), np.where(np.isfinite(want[pid]), 0, want[pid]))
+        finite = np.isfinite(want[pid])
+        check_grad(np.where(finite, g[pid], 0), np.where(finite, want[pid], 0), dims)
+    if where not in ("observations", "rewards"):
+        assert np.all(np.isfinite(g[1]))
