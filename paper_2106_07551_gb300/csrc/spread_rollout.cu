@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
     float4* buf = reinterpret_cast<float4*>(smem + SM::stage_at(groups) + (uint32_t)warp * SM::kStage);
     uint64_t* bar = bars[grp];
     uint32_t phase[2] = {0, 0};
+    uint32_t turn = 0;                                   // buffer of acts, alternating over units and items
     auto is_dead = [&] { return *(volatile uint32_t*)&dead != 0u; };
     auto group_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); };
     // layer `layer` (0, 1) of the group's current tile has completed
@@ -341,11 +342,12 @@ __global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
                 }
                 if (plan.share) {
                     // the other groups' actions (a buffer is written again only
-                    // after the next step's barrier)
-                    acts[t & 1][grp][r] = (uint16_t)act_pk;
+                    // after the next exchange's barrier, be it in the next unit)
+                    acts[turn][grp][r] = (uint16_t)act_pk;
                     asm volatile("bar.sync %0, %1;" ::"r"(kMaxGroups + 1), "r"((int)blockDim.x) : "memory");
                     for (int q = 0; q < groups; ++q)
-                        if (q != grp) act_pk |= acts[t & 1][q][r];
+                        if (q != grp) act_pk |= acts[turn][q][r];
+                    turn ^= 1u;
                 }
                 int act[N];
                 float rw[N];

@@ -53,3 +53,20 @@ def test_remote_shared_memory_waits_for_its_cta():
             assert arrive >= 0, f"{name}: no cluster barrier before the first remote access"
             assert any(c in before[arrive:] for c in call["wait"]), f"{name}: no wait before the first remote access"
     assert kernels == 2                  # Kuhn's clusters and the linear program's
+
+
+def test_action_buffers_alternate_across_units():
+    """Groups that share a unit exchange actions through two buffers with one barrier a
+    step, so successive exchanges must take different buffers also where one unit (of an
+    odd number of steps) ends and the next begins: the buffer comes from a variable that
+    is declared before the loop over items and flipped after each exchange."""
+    src = open(os.path.join(ROOT, "paper_2106_07551_gb300", "csrc", "spread_rollout.cu")).read()
+    body = src[src.index("spread_rollout_x3_kernel("):]
+    uses = re.findall(r"\bacts\[([^\]]*)\]\[", body)
+    uses.remove("2")                                     # the declaration
+    assert len(uses) == 2 and len(set(uses)) == 1
+    var = uses[0]
+    assert re.fullmatch(r"\w+", var), var
+    items = body.index("item < plan.items")
+    assert re.search(r"\b%s = 0;" % var, body[:items])
+    assert re.search(r"\b%s \^= 1u;" % var, body[body.rindex("acts["):])
