@@ -21,7 +21,9 @@ namespace {
 constexpr int kFpWarps = 8;                     // warps per side
 constexpr int kFpPer = 4;                       // rows (columns) per thread: m, n <= 1024
 constexpr int kFpMaxDim = 32 * kFpWarps * kFpPer;
-constexpr int kSmemLimit = 200 * 1024;          // bytes of payoff / tableau kept on chip
+// Bytes of payoff / tableau kept on chip; also the kernels' dynamic shared memory limit,
+// which is the process's, so that calls of several threads never lower one another's.
+constexpr int kSmemLimit = 200 * 1024;
 
 // Order-preserving integer key of a finite double (larger double, larger
 // key), and its inverse. The comparisons of a play run on these keys: fp64
@@ -482,7 +484,7 @@ cudaError_t launch_fictitious_play(const double* P, int32_t G, int32_t m, int32_
                            : fictitious_play_kernel<C, 1, 8>;
     };
     auto kern = on_chip ? pick_kernel(std::true_type{}) : pick_kernel(std::false_type{});
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<fp_grid(G, n_sm), 32 * (wr + wc), dyn, s>>>(P, G, m, n, stride, T, wr, x, y, bounds);
     return cudaGetLastError();
@@ -533,7 +535,7 @@ cudaError_t launch_lp_nash(const double* P, int32_t G, int32_t m, int32_t n, int
     const LpShape sh = lp_shape(G, m, n, stride, n_sm);
     const size_t dyn = sh.on_chip ? (size_t)sh.cta_doubles * 8 : 0;
     auto kern = sh.cluster > 1 ? lp_nash_kernel<true> : lp_nash_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(lp_grid(G, n_sm) * sh.cluster));

@@ -432,10 +432,11 @@ cudaError_t launch_rollout(const RolloutArgs& a, int n_sm, cudaStream_t s) {
     int64_t grid = 1;
     const RolloutPlan plan = rollout_plan(a.n_pairs, N, a.n_envs / a.n_pairs, a.n_episodes, n_sm, &groups, &grid);
     auto kern = a.logits ? spread_rollout_x3_kernel<N, IN, kScen, true> : spread_rollout_x3_kernel<N, IN, kScen, false>;
-    const uint32_t bytes = SM::bytes(groups);
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the limit is the process's: the most that any call takes, so that a call of another
+    // thread never lowers it between this one's two steps
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(kMaxGroups));
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)grid, kGroupThreads * groups, bytes, s>>>(a, plan);
+    kern<<<(unsigned)grid, kGroupThreads * groups, SM::bytes(groups), s>>>(a, plan);
     return cudaGetLastError();
 }
 
