@@ -177,48 +177,58 @@ __global__ void __launch_bounds__(64 * W) fictitious_play_kernel(
 }
 
 // Payoffs under a pair of mixtures: A y (per row), x^T A (per column), x^T A y.
-// One block per game. Rows: a warp each, lanes over the columns. Columns: a
-// lane each, the rows dealt over the warps of its column group, their partial
-// sums combined in warp order. 64 x 64 with stride 4: 13 us (a thread per row and
-// column, uncoalesced rows: 23).
-constexpr int kAggThreads = 512, kAggWarps = kAggThreads / 32;
-
-__global__ void __launch_bounds__(kAggThreads) aggregate_kernel(
-    const double* __restrict__ P, int32_t n_games, int32_t m, int32_t n, int32_t stride,
+// One block of W warps per game. Rows: kRowLanes lanes each over the columns (32 /
+// kRowLanes rows of a warp at once). Columns: a lane each, the rows dealt over the
+// warps of its column group. kRowLanes = 0 is for narrow tables, `lanes` (the columns,
+// rounded up to a power of two) at most 16: up to 4 lanes a row, and in the second
+// pass 32 / lanes rows of a warp at once. Partial sums are combined in a fixed order.
+template <int W, int kRowLanes>
+__global__ void __launch_bounds__(32 * W) aggregate_kernel(
+    const double* __restrict__ P, int32_t n_games, int32_t m, int32_t n, int32_t stride, int32_t lanes,
     const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ ay_out,
     double* __restrict__ xa_out, double* __restrict__ val_out) {
-    __shared__ double red[kAggWarps];
-    __shared__ double col[kAggWarps][32];
+    __shared__ double red[W];
+    __shared__ double col[W][32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int L = kRowLanes ? kRowLanes : min(lanes, 4);         // lanes of a row, first pass
+    const int C = kRowLanes ? 32 : lanes;                        // columns of a warp, second pass
     for (int g = blockIdx.x; g < n_games; g += gridDim.x) {
         const double* Pg = P + (int64_t)g * m * n * stride;
         const double* xg = x + (int64_t)g * m;
         const double* yg = y + (int64_t)g * n;
-        double part = 0.0;                       // of x^T A y: this warp's rows, in row order
-        for (int i = warp; i < m; i += kAggWarps) {
+        double part = 0.0;                       // of x^T A y: this lane group's rows, in row order
+        for (int i0 = warp * (32 / L); i0 < m; i0 += W * (32 / L)) {
+            const int i = i0 + lane / L;
             double s = 0.0;
+            if (i < m)
 #pragma unroll 4
-            for (int j = lane; j < n; j += 32) s = fma(Pg[((int64_t)i * n + j) * stride], yg[j], s);
+                for (int j = lane & (L - 1); j < n; j += L) s = fma(Pg[((int64_t)i * n + j) * stride], yg[j], s);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) ay_out[(int64_t)g * m + i] = s;
-            part = fma(xg[i], s, part);
+            for (int o = 16; o > 0; o >>= 1)
+                if (o < L) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (i < m) {
+                if ((lane & (L - 1)) == 0) ay_out[(int64_t)g * m + i] = s;
+                part = fma(xg[i], s, part);
+            }
         }
+        for (int o = L; o < 32; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         if (lane == 0) red[warp] = part;
-        // columns, 32 groups of columns at a time over all warps
+        // columns, W groups of them at a time over all warps
         const int groups = (n + 31) / 32;
-        for (int c0 = 0; c0 < groups; c0 += kAggWarps) {
-            const int here = min(kAggWarps, groups - c0);        // column groups of this round
-            const int per = kAggWarps / here;                    // warps per group
+        for (int c0 = 0; c0 < groups; c0 += W) {
+            const int here = min(W, groups - c0);                // column groups of this round
+            const int per = W / here;                            // warps per group
             const int grp = warp / per, sub = warp - grp * per;
-            const int j = (c0 + grp) * 32 + lane;
+            const int j = (c0 + grp) * 32 + (lane & (C - 1));
             double s = 0.0;
             if (grp < here && j < n)
 #pragma unroll 4
-                for (int i = sub; i < m; i += per) s = fma(xg[i], Pg[((int64_t)i * n + j) * stride], s);
+                for (int i = sub * (32 / C) + lane / C; i < m; i += per * (32 / C))
+                    s = fma(xg[i], Pg[((int64_t)i * n + j) * stride], s);
+            for (int o = C; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             col[warp][lane] = s;
             __syncthreads();
-            if (grp < here && sub == 0 && j < n) {
+            if (grp < here && sub == 0 && lane < C && j < n) {
                 for (int q = 1; q < per; ++q) s += col[warp + q][lane];
                 xa_out[(int64_t)g * n + j] = s;
             }
@@ -226,7 +236,7 @@ __global__ void __launch_bounds__(kAggThreads) aggregate_kernel(
         }
         if (tid == 0) {
             double v = 0.0;
-            for (int w = 0; w < kAggWarps; ++w) v += red[w];
+            for (int w = 0; w < W; ++w) v += red[w];
             val_out[g] = v;
         }
         __syncthreads();
@@ -493,7 +503,29 @@ cudaError_t launch_fictitious_play(const double* P, int32_t G, int32_t m, int32_
 cudaError_t launch_aggregate(const double* P, int32_t G, int32_t m, int32_t n, int32_t stride,
                              const double* x, const double* y, double* ay, double* xa, double* val,
                              int n_sm, cudaStream_t s) {
-    aggregate_kernel<<<fp_grid(G, n_sm), kAggThreads, 0, s>>>(P, G, m, n, stride, x, y, ay, xa, val);
+    int32_t lanes = 1;
+    while (lanes < n && lanes < 32) lanes *= 2;
+    // Small tables come many at a time: fewer warps a game, more games at once (16
+    // warps and a warp per row throughout: 10,000 games 2 x 2 91 us, 60 x 10 409, 45 x 45
+    // 421; a thread per row and column in 8 warps: 44, 129, 375; so: 19, 72, 198). Wide
+    // rows want all lanes; others share a warp, whose fp64 pipe (2 lanes a clock and SM)
+    // would otherwise spend five additions a row on combining lanes (one game 100 x 100
+    // 12.6 us, 32 lanes a row 20.5; 2,000 x 2,000 4,160 us with 8 lanes, 2,910 with 32).
+    const int64_t size = (int64_t)m * n;
+    void (*kern)(const double*, int32_t, int32_t, int32_t, int32_t, int32_t, const double*, const double*, double*,
+                 double*, double*);
+    const int W = n > 256 || size > 4096 ? 16 : size > 1024 ? 8 : size > 256 ? 4 : 2;
+    if (lanes <= 16)
+        kern = W == 2 ? aggregate_kernel<2, 0> : W == 4 ? aggregate_kernel<4, 0> : W == 8 ? aggregate_kernel<8, 0>
+                                                                                 : aggregate_kernel<16, 0>;
+    else
+        kern = n > 256  ? aggregate_kernel<16, 32>
+               : W == 2 ? aggregate_kernel<2, 8>
+               : W == 4 ? aggregate_kernel<4, 8>
+               : W == 8 ? aggregate_kernel<8, 8>
+                        : aggregate_kernel<16, 8>;
+    const int64_t most = (int64_t)n_sm * (W == 2 ? 32 : 64 / W);               // resident blocks
+    kern<<<(unsigned)(G < most ? G : most), 32 * W, 0, s>>>(P, G, m, n, stride, lanes, x, y, ay, xa, val);
     return cudaGetLastError();
 }
 

@@ -243,6 +243,29 @@ def test_aggregate(ctx):
         assert abs(float(val[g]) - r_v) <= 1e-12 * s * (m + n)
 
 
+@pytest.mark.parametrize("G,m,n", [(3, 1, 1), (5000, 2, 2), (2, 7, 16), (2, 15, 17), (2, 16, 16), (2, 17, 16), (2, 60, 10),
+                                   (2, 100, 13), (2, 300, 16), (2, 3, 65), (2, 32, 32), (2, 33, 33), (700, 45, 70),
+                                   (2, 64, 64), (2, 70, 70), (2, 20, 256), (2, 5, 257), (1, 3, 1000), (1, 2000, 1)])
+def test_aggregate_shapes(ctx, G, m, n):
+    """Both sides of the dispatch: tables of up to 256, 1,024, 4,096 and more entries, up to
+    16, 256 and more columns, more games than resident blocks; entry 0 of 4. The bound is
+    that of fp64 sums of m, n or m n terms in any order."""
+    torch = need_gpu()
+    rng = np.random.default_rng(m * n)
+    raw = rng.normal(size=(G, m, n, 4))
+    x, y = rng.dirichlet(np.ones(m), size=G), rng.dirichlet(np.ones(n), size=G)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    ay, xa, val = (torch.full(s, np.nan, dtype=torch.float64, device="cuda") for s in ((G, m), (G, n), (G,)))
+    ctx.meta_aggregate(d(raw), d(x), d(y), ay, xa, val, stride=4)
+    ctx.sync()
+    A, u = raw[..., 0], 2.0 ** -53
+    size = [np.einsum(e, *o) for e, o in (("gij,gj->gi", (abs(A), y)), ("gi,gij->gj", (x, abs(A))),
+                                          ("gi,gij,gj->g", (x, abs(A), y)))]
+    for got, want, s, terms in ((ay, np.einsum("gij,gj->gi", A, y), size[0], n), (xa, np.einsum("gi,gij->gj", x, A), size[1], m),
+                                (val, np.einsum("gi,gij,gj->g", x, A, y), size[2], m + n)):
+        assert np.all(np.abs(got.cpu().numpy() - want) <= 2 * (terms + 2) * u * s)
+
+
 def test_errors(ctx):
     torch = need_gpu()
     from paper_2106_07551_gb300 import MalibError
