@@ -91,11 +91,19 @@ __device__ __forceinline__ Cand warp_best(Cand a) {
 // argmax by 64-bit shuffles and the candidates reduced again in every warp 575.
 // Warps 0 .. wr - 1 hold the rows (row lane + 32 w + 32 wr k), the rest the
 // columns. K: rows (columns) per thread; W: candidates per side read (1, 2, 4, 8).
-template <bool kOnChip, int K, int W>
+// kTable: the payoffs on chip, or read where they lie with strides that fit 32 bits (a
+// 64-bit product is on the chain of a play: 1 % at 256 x 256), or with any.
+enum FpTable { kFpOnChip, kFpNear, kFpFar };
+template <FpTable kTable, int K, int W>
 __global__ void __launch_bounds__(64 * W) fictitious_play_kernel(
     const double* __restrict__ P, int32_t n_games, int32_t m, int32_t n, int32_t stride,
     int64_t T, int32_t wr, double* __restrict__ x_out, double* __restrict__ y_out,
     double* __restrict__ bounds_out) {
+    constexpr bool kOnChip = kTable == kFpOnChip;
+    // This side's best while the payoffs arrive (256 x 256: 797 -> 769 ns a play), where
+    // they come from L2; from shared memory at once with the other's (64 x 64: 348 -> 328
+    // us for 2,000 plays), and with four rows a thread too (513 x 513: 1,183 -> 1,120 ns).
+    constexpr bool kOwnLate = !kOnChip && K <= 2;
     extern __shared__ double sA[];              // [m][ld] when on chip
     __shared__ Cand red[2][2][W];               // [play's parity][side][warp]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -129,40 +137,44 @@ __global__ void __launch_bounds__(64 * W) fictitious_play_kernel(
             at[k] = (kOnChip ? sA : Pg) + (q < dim ? q * sq : 0);
         }
         int other = 0, own = 0;
-        Cand best_own{kNone, 0}, best_other{kNone, 0};
+        // the best of the other side's candidates (of == 1) or of this side's (of == 0)
+        auto best_of = [&](int par, int of) {
+            Cand c[W];
+#pragma unroll
+            for (int q = 0; q < W; ++q) c[q] = red[par][side ^ of][q];
+#pragma unroll
+            for (int h = W / 2; h > 0; h >>= 1)
+#pragma unroll
+                for (int q = 0; q < h; ++q) c[q] = pick(c[q], c[q + h]);
+            return c[0];
+        };
+        Cand best_other{kNone, 0};
         for (int64_t t = 0; t < T; ++t) {
             const int par = (int)(t & 1);
             Cand b{kNone, 0x7fffffff};
+            double a[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                a[k] = kOnChip             ? at[k][other * (int)so]
+                       : kTable == kFpNear ? __ldg(at[k] + (int64_t)other * (int)so)
+                                           : __ldg(at[k] + other * so);
+            if (kOwnLate && t > 0) own = best_of(par ^ 1, 0).i;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 const int q = lane + 32 * (w + ws * k);
-                const double a = kOnChip ? at[k][other * (int)so] : __ldg(at[k] + other * so);
                 cnt[k] += q == own ? 1 : 0;
-                u[k] += a;
+                u[k] += a[k];
                 const long long key = side ? -okey(u[k]) : okey(u[k]);
                 if (q < dim) b = pick(b, Cand{key, q});
             }
             b = warp_best(b);
             if (lane == 0) red[par][side][w] = b;
             __syncthreads();
-            Cand c[2][W];
-#pragma unroll
-            for (int q = 0; q < W; ++q) {
-                c[0][q] = red[par][side ^ 1][q];
-                c[1][q] = red[par][side][q];
-            }
-#pragma unroll
-            for (int h = W / 2; h > 0; h >>= 1)
-#pragma unroll
-                for (int q = 0; q < h; ++q) {
-                    c[0][q] = pick(c[0][q], c[0][q + h]);
-                    c[1][q] = pick(c[1][q], c[1][q + h]);
-                }
-            best_other = c[0][0];
-            best_own = c[1][0];
+            best_other = best_of(par, 1);
             other = best_other.i;
-            own = best_own.i;
+            if (!kOwnLate) own = best_of(par, 0).i;
         }
+        const Cand best_own = best_of((int)((T - 1) & 1), 0);
         const double Td = (double)T;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -485,15 +497,18 @@ cudaError_t launch_fictitious_play(const double* P, int32_t G, int32_t m, int32_
     auto warps = [&](int d) { return (d + 32 * per - 1) / (32 * per); };
     const int wr = warps(m), wc = warps(n);
     const int most = wr > wc ? wr : wc;
-    auto pick_kernel = [&](auto chip) {
-        constexpr bool C = decltype(chip)::value;
-        return per > 1     ? fictitious_play_kernel<C, kFpPer, 8>
-               : most <= 1 ? fictitious_play_kernel<C, 1, 1>
-               : most <= 2 ? fictitious_play_kernel<C, 1, 2>
-               : most <= 4 ? fictitious_play_kernel<C, 1, 4>
-                           : fictitious_play_kernel<C, 1, 8>;
+    auto pick_kernel = [&](auto where) {
+        constexpr FpTable T = decltype(where)::value;
+        return per > 2     ? fictitious_play_kernel<T, kFpPer, 8>
+               : per > 1   ? fictitious_play_kernel<T, 2, 8>     // (fp64 additions of absent rows cost as much as others)
+               : most <= 1 ? fictitious_play_kernel<T, 1, 1>
+               : most <= 2 ? fictitious_play_kernel<T, 1, 2>
+               : most <= 4 ? fictitious_play_kernel<T, 1, 4>
+                           : fictitious_play_kernel<T, 1, 8>;
     };
-    auto kern = on_chip ? pick_kernel(std::true_type{}) : pick_kernel(std::false_type{});
+    auto kern = on_chip ? pick_kernel(std::integral_constant<FpTable, kFpOnChip>{})
+                : (int64_t)stride * n <= INT32_MAX ? pick_kernel(std::integral_constant<FpTable, kFpNear>{})
+                                                   : fictitious_play_kernel<kFpFar, kFpPer, 8>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<fp_grid(G, n_sm), 32 * (wr + wc), dyn, s>>>(P, G, m, n, stride, T, wr, x, y, bounds);

@@ -72,6 +72,9 @@ def test_fp_bit_exact_off_chip_and_max(ctx):
     check_fp_exact(t3, 120, *run_fp(ctx, t3, 120))
     t4 = rng.normal(size=(2, 257, 100))             # 257 rows: two per thread for some
     check_fp_exact(t4, 120, *run_fp(ctx, t4, 120))
+    for m, n in ((512, 40), (40, 512), (513, 40)):  # two and three rows per thread
+        t5 = rng.normal(size=(1, m, n))
+        check_fp_exact(t5, 120, *run_fp(ctx, t5, 120))
 
 
 def test_fp_many_games(ctx):
