@@ -85,7 +85,8 @@ __device__ __forceinline__ void kuhn_hands(const EvalArgs& a, int pair, int p0, 
     }
 }
 
-__global__ void __launch_bounds__(256) kuhn_eval_kernel(EvalArgs a) {
+// (four blocks on an SM: with 72 registers a thread three were, 992 pairs x 3,073 hands 47 -> 51 us)
+__global__ void __launch_bounds__(256, 4) kuhn_eval_kernel(EvalArgs a) {
     const int pair = blockIdx.y;
     const int p0 = a.pairs[2 * pair], p1 = a.pairs[2 * pair + 1];
     const bool ok = pair_ok(a, p0, p1);
@@ -108,8 +109,8 @@ __global__ void __launch_bounds__(256) kuhn_eval_kernel(EvalArgs a) {
     }
 }
 
-// The same with a cluster per pair: the CTAs' sums (32-bit: at most 4 hands a
-// thread) meet in the first one's shared memory, which writes the pair's row and
+// The same with a cluster per pair: the CTAs' sums (32-bit: at most 3,072 hands a
+// CTA) meet in the first one's shared memory, which writes the pair's row and
 // its decision count. No accumulators in global memory to clear, add to and count
 // blocks with: a table of 16 pairs x 10,000 hands is bound by latencies (the
 // policies' loads, two hands a thread, the fp64 division and square root of the
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(kKuhnMaxThreads, 2) kuhn_cluster_kernel(EvalAr
 }
 
 // CTAs per pair of kuhn_cluster_kernel; 0: kuhn_eval_kernel takes the call. A pair's
-// cluster of at most 8 CTAs plays up to 4 hands a thread; longer calls are bound by
+// cluster of at most 8 CTAs plays up to 3,072 hands a CTA; longer calls are bound by
 // the generator and go over all the SMs. Both sides, in us a call (clusters, blocks):
 // 1 x 2,000 hands 6.2, 9.2; 1 x 24,000 10.3, 10.3; 16 x 24,000 14.9, 16.5;
 // 64 x 24,000 26.7, 28.8; 256 x 6,000 (2 CTAs a pair) 26.7, 28.8; 1,000 x 3,000 41, 44.
@@ -207,7 +208,12 @@ cudaError_t launch_kuhn_eval(const EvalArgs& a, int n_sm, cudaStream_t s) {
     if (a.n_pairs == 0) return cudaSuccess;
     if (const int c = a.fin_out ? kuhn_cluster(a.n_pairs, a.n_episodes, n_sm) : 0) {
         const int64_t per = (a.n_episodes + c - 1) / c;                      // hands of a CTA
-        const int64_t turns = (per + kKuhnMaxThreads - 1) / kKuhnMaxThreads;
+        // Few CTAs: as many threads as there are, one hand each (latency). More than two an
+        // SM: blocks of 256, so that one's last steps (a row's fp64 division and root)
+        // overlap others' hands; 40,000 pairs x 768 hands 705 -> 344 us, x 2,000 1,076 -> 817
+        // (kuhn_eval_kernel 490, 911)
+        const int64_t most = (int64_t)a.n_pairs * c >= 2 * (int64_t)n_sm ? 256 : kKuhnMaxThreads;
+        const int64_t turns = (per + most - 1) / most;
         cudaLaunchAttribute attr{};
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = (unsigned)c;

@@ -102,7 +102,7 @@ def test_device_buffers_and_determinism(kuhn_ctx):
 
 
 @pytest.mark.parametrize("n_pairs,n_eps", [(1, 1), (1, 127), (1, 128), (16, 24576), (16, 24577), (76, 6145), (77, 12288),
-                                           (77, 12289), (153, 6144), (305, 3072), (305, 3073)])
+                                           (77, 12289), (153, 6144), (305, 3072), (305, 3073), (400, 300)])
 def test_table_sums_on_both_sides_of_the_cluster_rule(kuhn_ctx, orc, n_pairs, n_eps):
     """A cluster of 8, 4, 2 or 1 CTAs per pair up to 3,072 hands a CTA, blocks adding to global
     accumulators past it: the integer sums and the decision count equal the oracle's."""
