@@ -31,6 +31,7 @@
 #include "internal.h"
 #include "leduc_env.cuh"
 #include "mlp_tc2.cuh"
+#include "segments.h"
 
 namespace malib {
 
@@ -454,28 +455,16 @@ int64_t leduc_tc_units(int32_t n_pairs, int64_t n_episodes, int n_sm, int64_t* n
                        int32_t* split_from_out) {
     int64_t n_seg = (n_episodes + kLeducTcMaxHands - 1) / kLeducTcMaxHands;
     if (n_pairs <= n_sm) {
-        // few pairs: the number of segments with the smallest estimated time. A
-        // unit's phase costs about 5 us and 2.2 us a tile, and of its hands about
-        // these shares act in its phases; the units go over the SMs in waves. (65
-        // pairs x 2,000 hands: 3 segments, enough for every SM, made 195 units and
-        // two waves, 216 us a call; 2 segments make one, 159.)
-        static const double share[8] = {1.0, 1.0, 0.8, 0.6, 0.4, 0.25, 0.1, 0.05};
+        // few pairs: the number of segments with the smallest estimated time (a
+        // unit's phase costs about 5 us, and 2.2 us a tile of 128 hands). (65 pairs x
+        // 2,000 hands: 3 segments, enough for every SM, made 195 units and two waves,
+        // 216 us a call; 2 segments make one, 159.)
         const int64_t lo = n_seg, most = (n_episodes + 127) / 128;
         int64_t hi = 3 * (int64_t)n_sm / n_pairs + 2;
         if (hi < 4 * lo) hi = 4 * lo;
         if (hi > most) hi = most > lo ? most : lo;
         if (hi > lo + 4096) hi = lo + 4096;
-        double best = 1e300;
-        for (int64_t seg = lo; seg <= hi; ++seg) {
-            const int64_t per = (n_episodes + seg - 1) / seg;
-            double cost = 0.0;
-            for (double sh : share) cost += 5.0 + 2.2 * (double)(int64_t)((double)per * sh / 128.0 + 0.999);
-            cost *= (double)(((int64_t)n_pairs * seg + n_sm - 1) / n_sm);
-            if (cost < best) {
-                best = cost;
-                n_seg = seg;
-            }
-        }
+        n_seg = cheapest_segments(n_pairs, n_episodes, n_sm, lo, hi, 5.0, 2.2, 128.0);
     }
     // when there are more pairs than SMs, the last n_sm pairs (the last units
     // claimed) are played in halves: a unit's time varies with its policies,

@@ -49,6 +49,7 @@
 #include "internal.h"
 #include "leduc_env.cuh"
 #include "mlp_x3.cuh"
+#include "segments.h"
 
 namespace malib {
 
@@ -541,29 +542,15 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
 }
 
 // Segments per pair: the smallest estimated time. A unit's phase costs a policy
-// conversion and the first tile's chain, and each further pair of tiles a chain;
-// of a unit's hands, about these shares act in its phases.
+// conversion and the first tile's chain (4 us), and each pair of tiles a chain (6).
 LeducUnits plan_units(int32_t n_pairs, int64_t n, int n_sm) {
-    static const double share[8] = {1.0, 1.0, 0.8, 0.6, 0.4, 0.25, 0.1, 0.05};
     const int64_t lo = (n + kMaxHands - 1) / kMaxHands;
     int64_t hi = 2 * (int64_t)n_sm / n_pairs + 2;            // up to two waves of units
     if (hi < 4 * lo) hi = 4 * lo;
     if (hi > (n + 63) / 64) hi = (n + 63) / 64 > lo ? (n + 63) / 64 : lo;
     if (hi > lo + 4096) hi = lo + 4096;
-    LeducUnits best{};
-    double best_cost = 1e300;
-    for (int64_t seg = lo; seg <= hi; ++seg) {
-        const int64_t per = (n + seg - 1) / seg;
-        const double turns = (double)(((int64_t)n_pairs * seg + n_sm - 1) / n_sm);
-        double cost = 0.0;
-        for (double sh : share) cost += 4.0 + 6.0 * (double)(int64_t)((double)per * sh / 256.0 + 0.999);
-        cost *= turns;
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = LeducUnits{seg, per, (int64_t)n_pairs * seg};
-        }
-    }
-    return best;
+    const int64_t seg = cheapest_segments(n_pairs, n, n_sm, lo, hi, 4.0, 6.0, 256.0);
+    return LeducUnits{seg, (n + seg - 1) / seg, (int64_t)n_pairs * seg};
 }
 
 template <int H>
