@@ -7,8 +7,9 @@
 // Work units are (pair, segment of at most kMaxHands hands), claimed by the CTAs
 // from a counter. A CTA plays a unit's hands all at once, in phases: in a phase
 // every live hand whose acting seat is s makes one decision through seat s's
-// policy, the only one in shared memory; phases alternate between the seats and
-// the policy is converted from the population's fp32 image between them. Hands
+// policy; phases alternate between the seats. Policies are converted from the
+// population's fp32 images: 128 wide only the acting seat's fits in shared memory,
+// between the phases, 64 wide both seats' stay until a unit has others. Hands
 // live in shared memory: a 27-bit state word each, and a list of hand numbers per
 // acting seat. A phase takes its seat's list whole; hands that act next as the
 // other seat join the other list, hands that act again as s a third one, which
@@ -74,24 +75,26 @@ struct LeducX3 {
     __host__ __device__ static constexpr uint32_t hid_col(int b, int part) {
         return (b < H / 64 ? 3u * H / 4 + 48u * b : 48u * (b - H / 64)) + 16u * part;
     }
-    // shared memory (bytes)
+    // shared memory (bytes): the policies (64 wide, both seats'; 128 wide, the acting seat's)
+    static constexpr int kPols = H == 64 ? 2 : 1;
     static constexpr uint32_t kLboX = 128 / 8 * 128, kLboW = H / 8 * 128;
     static constexpr uint32_t kStep = 2 * kLboW;               // one K = 16 step of a weight image
     static constexpr uint32_t kPart2 = (uint32_t)H * H * 2;
     static constexpr uint32_t kW2 = 0;                         // parts h, m, l
     static constexpr uint32_t kW1 = kW2 + 3 * kPart2;          // steps [wh 2][wm 2][wl 1]
     static constexpr uint32_t kB2 = kW1 + 5 * kStep;           // bias step [H][16]
-    static constexpr uint32_t kOnes = kB2 + kStep;             // [128][16] rows 1 1 1 0 ..
+    static constexpr uint32_t kW3 = kB2 + kStep;               // fp32 [3][H], b3
+    static constexpr uint32_t kPolicy = (kW3 + (3 * H + 4) * 4 + 127) / 128 * 128;
+    static constexpr uint32_t kOnes = kPols * kPolicy;         // [128][16] rows 1 1 1 0 ..
     static constexpr uint32_t kXBytes = 128 * 32 * 2;
     static constexpr uint32_t kX = kOnes + 128 * 16 * 2;
-    static constexpr uint32_t kW3 = kX + kGroups * kXBytes;    // fp32 [3][H], b3
-    static constexpr uint32_t kP = kW3 + (3 * H + 4) * 4;      // partial logits [group][128] float4
+    static constexpr uint32_t kP = kX + kGroups * kXBytes;     // partial logits [group][128] float4
     static constexpr uint32_t kState = kP + kGroups * 128 * 16;
     static constexpr uint32_t kList = kState + kMaxHands * 4;  // uint16 [3][kMaxHands]
     static constexpr uint32_t kBytes = kList + 3 * kMaxHands * 2;
     static_assert(kBytes + 1280 <= 232448, "fits the 227 KB of shared memory of a CTA");
 
-    // Converts a policy (fp32 image in global memory) into shared memory; all
+    // Converts a policy (fp32 image in global memory) into shared memory at sm; all
     // threads, the caller fences for the async proxy and synchronises.
     __device__ static void stage(uint8_t* sm, const float* __restrict__ src, int tid) {
         // W2: a thread converts 8 k of one row at a time (coalesced loads, 16-byte stores)
@@ -191,15 +194,15 @@ struct LeducX3 {
         tc::mma_commit(bar);
     }
 
-    // One elected thread: layer 2's output units 64 n .. into D2.
-    __device__ static void issue2(uint32_t tb, uint32_t sm, int n, uint64_t* bar) {
+    // One elected thread: layer 2's output units 64 n .. into D2 (sm: the policy's).
+    __device__ static void issue2(uint32_t tb, uint32_t sm, uint32_t ones, int n, uint64_t* bar) {
         const uint32_t idesc = tc::instr_desc(128, 64, 1);
         const uint64_t w = tc::smem_desc(sm + kW2 + 1024u * n, kLboW, 128);
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
             const int px = q == 0 ? 2 : (q == 1 || q == 3) ? 1 : 0, pw = q == 2 ? 2 : (q == 1 || q == 4) ? 1 : 0;
             if (q == 5)
-                tc::mma_bf16(tb + kD2, tc::smem_desc(sm + kOnes, kLboX, 128),
+                tc::mma_bf16(tb + kD2, tc::smem_desc(ones, kLboX, 128),
                              tc::smem_desc(sm + kB2 + 1024u * n, kLboW, 128), idesc, true);
 #pragma unroll
             for (int k = 0; k < H / 16; ++k)
@@ -312,7 +315,6 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
     float4* P = reinterpret_cast<float4*>(smem + E::kP) + 128 * grp;
     uint32_t* state = reinterpret_cast<uint32_t*>(smem + E::kState);
     uint16_t* lists = reinterpret_cast<uint16_t*>(smem + E::kList);
-    const float* b3 = reinterpret_cast<const float*>(smem + E::kW3) + 3 * H;
     uint64_t* bar = bars[grp];
     uint32_t phase_bit = 0;                // the group's tiles so far, mod 2
     auto is_dead = [&] { return *(volatile uint32_t*)&dead != 0u; };
@@ -325,7 +327,8 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
         }
         tc::fence_after_sync();
     };
-    int staged = -1;
+    long long nd = 0;                      // this thread's decisions
+    int staged[2] = {-1, -1};              // the policies in shared memory
 
     while (true) {
         __syncthreads();                                     // unit_s and len are read by all
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
         }
         if (n_hands == 0) continue;
         const uint64_t g0 = (uint64_t)pair * (uint64_t)a.n_episodes + (uint64_t)e_lo;
-        long long s1 = 0, s2 = 0, nd = 0;
+        int s1 = 0, s2 = 0;                                  // of at most 8,192 hands
         int mine[2] = {0, 1}, spare = 2;                     // the seats' lists, and the third
         bool first = true;                                   // the phase that deals the hands
         for (int s = 0;; s ^= 1) {
@@ -359,10 +362,12 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                 if (n0 == 0 && n1 == 0) break;
                 continue;
             }
-            const int pol = pid[s];
-            if (pol != staged) {
-                E::stage(smem, a.arena + a.pol_offset[pol], tid);
-                staged = pol;
+            const int pol = pid[s], at = E::kPols == 2 ? s : 0;
+            uint8_t* const ps = smem + (uint32_t)at * E::kPolicy;
+            const uint32_t pu = smem_u32(ps);
+            if (pol != (at ? staged[1] : staged[0])) {
+                E::stage(ps, a.arena + a.pol_offset[pol], tid);
+                (at ? staged[1] : staged[0]) = pol;
             }
             fence_proxy_async_smem();
             __syncthreads();                                 // also: everyone has read len
@@ -407,7 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                 tc::fence_before_sync();
                 group_sync();
                 tc::fence_after_sync();
-                if (issuer && !is_dead() && tc::elect_one()) E::issue1(tb, smem_u32(smem), smem_u32(X), bar);
+                if (issuer && !is_dead() && tc::elect_one()) E::issue1(tb, pu, smem_u32(X), bar);
                 __syncwarp();
             }
             for (int i = grp; i < tiles; i += kGroups) {
@@ -420,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                     tc::fence_before_sync();
                     group_sync();                            // HID is written; D2 is read
                     tc::fence_after_sync();
-                    if (issuer && !is_dead() && tc::elect_one()) E::issue2(tb, smem_u32(smem), p, bar + 1 + p);
+                    if (issuer && !is_dead() && tc::elect_one()) E::issue2(tb, pu, smem_u32(smem + E::kOnes), p, bar + 1 + p);
                     __syncwarp();
                     if (hh == 0) {
                         if (p == 0 && id >= 0) u = u24(draw(g0 + (uint64_t)id, (w >> 15) & 15u, (uint32_t)s, a.seed).x);
@@ -430,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                         }
                     }
                     mma_wait(1 + p);
-                    E::logits(tb, lane_q, smem, p, hh, acc);
+                    E::logits(tb, lane_q, ps, p, hh, acc);
                 }
                 float lg[3];
 #pragma unroll
@@ -444,10 +449,11 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                 tc::fence_after_sync();
                 phase_bit ^= 1u;
                 if (i + kGroups < tiles) {
-                    if (issuer && !is_dead() && tc::elect_one()) E::issue1(tb, smem_u32(smem), smem_u32(X), bar);
+                    if (issuer && !is_dead() && tc::elect_one()) E::issue1(tb, pu, smem_u32(X), bar);
                     __syncwarp();
                 }
                 if (hh == 0) {
+                    const float* b3 = reinterpret_cast<const float*>(ps + E::kW3) + 3 * H;
                     int next = -1;
                     if (id >= 0) {
                         const float4 o = P[r];
@@ -491,7 +497,7 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                         ++nd;
                         if (h.done) {
                             s1 += h.payoff;
-                            s2 += (long long)h.payoff * h.payoff;
+                            s2 += h.payoff * h.payoff;
                             if (rec) {
                                 for (int k = t; k < kMaxDec; ++k) {
                                     if (a.d_obs)
@@ -534,8 +540,17 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
             spare = done_list;
             first = false;
         }
-        block_add_sums(s1, s2, nd, a.acc + 2 * pair, a.n_dec);
+        if (hh == 0) {                                       // (integers: exact in any order)
+            s1 = __reduce_add_sync(0xffffffffu, s1);
+            s2 = __reduce_add_sync(0xffffffffu, s2);
+            if (lane == 0 && s2 != 0) {
+                atomicAdd(a.acc + 2 * pair, (u64)(long long)s1);
+                atomicAdd(a.acc + 2 * pair + 1, (u64)(long long)s2);
+            }
+        }
     }
+    nd = warp_sum_ll(nd);
+    if (lane == 0 && nd != 0) atomicAdd(a.n_dec, (u64)nd);
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem_base, 512);
