@@ -140,21 +140,6 @@ __device__ __forceinline__ void mbar_arrive_release(uint64_t* bar) {
                  : "memory");
 }
 
-// Shared -> global bulk copy (16-byte aligned addresses, size a multiple of
-// 16), tracked by the issuing thread's bulk groups.
-__device__ __forceinline__ void bulk_s2g(void* dst_gmem, const void* src_smem, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst_gmem),
-                 "r"(smem_u32(src_smem)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// The issuing thread's committed bulk copies have finished reading shared memory.
-__device__ __forceinline__ void bulk_wait_read() {
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// The issuing thread's committed bulk copies have completed.
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes,
                                          uint64_t* bar) {
     asm volatile(
@@ -191,30 +176,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 }
 
 constexpr uint64_t kWaitLimitNs = 1000000000ull;   // 1 s: far above any staging copy
-
-// Stages `bytes` (16-byte multiple) from global to shared with one elected
-// thread issuing bulk copies of at most 64 KB each; every thread then waits on
-// the barrier phase `parity` (bounded). On expiry raises ERRBIT_TIMEOUT,
-// waits once more (bounded) for the copies in flight, and returns false.
-__device__ __forceinline__ bool stage_to_smem(void* dst, const void* src, uint32_t bytes,
-                                              uint64_t* bar, uint32_t parity, int* err) {
-    if (threadIdx.x == 0) {
-        fence_proxy_async_smem();
-        mbar_arrive_expect_tx(bar, bytes);
-        uint32_t off = 0;
-        while (off < bytes) {
-            const uint32_t n = (bytes - off) < 65536u ? (bytes - off) : 65536u;
-            bulk_g2s((char*)dst + off, (const char*)src + off, n, bar);
-            off += n;
-        }
-    }
-    if (!mbar_wait_bounded(bar, parity, kWaitLimitNs)) {
-        atomicOr(err, ERRBIT_TIMEOUT);
-        mbar_wait_bounded(bar, parity, kWaitLimitNs);
-        return false;
-    }
-    return true;
-}
 
 // Warp-level inclusive sum helpers.
 __device__ __forceinline__ long long warp_sum_ll(long long v) {

@@ -50,19 +50,6 @@ __device__ __forceinline__ Cand pick(Cand a, Cand b) {
     return Cand{take ? b.k : a.k, take ? b.i : a.i};
 }
 
-template <int kSteps>
-__device__ __forceinline__ Cand warp_pick(Cand a) {
-#pragma unroll
-    for (int s = 0; s < kSteps; ++s) {
-        const int o = 1 << s;                   // butterfly over lane bits 0 .. kSteps-1
-        Cand b;
-        b.k = __shfl_xor_sync(0xffffffffu, a.k, o);
-        b.i = __shfl_xor_sync(0xffffffffu, a.i, o);
-        a = pick(a, b);
-    }
-    return a;
-}
-
 // The best candidate of a warp (every lane gets it): the largest key by its high
 // then its low word, then the lowest index, each one warp-wide integer
 // reduction. Five rounds of 64-bit shuffles and selects took about twice as long.
