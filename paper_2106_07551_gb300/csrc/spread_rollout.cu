@@ -24,7 +24,7 @@
 //
 // What bounds it: the chain of a tile through its group (about 5,000 cycles:
 // conversion 900, layer 2 1,000, logits 800, observation and stores 1,100, draw
-// 300), overlapped by three groups a CTA; tensor pipe 24 % busy, issue 38 %.
+// 300), overlapped by three groups a CTA; tensor pipe 35 % busy, issue 48 %.
 // 256-row passes of packed fp32 FMAs before (61 % of the FMA pipe, one episode
 // pair per CTA): spread 4,096 environments x 10 episodes 1,343 us, now 355;
 // tag 9 x 125 environments x 3 episodes 990 us, now 275.
@@ -124,11 +124,36 @@ __device__ __forceinline__ void scenario_obs(const Env& s, int i, float* o) {
     else spread_obs<N, XS>(s, i, o);
 }
 
+// The actions an agent may take.
+template <int kScen>
+__device__ __forceinline__ unsigned legal_of(int i) {
+    return (kScen == kSpeakerListener && i == 0) ? kSlSpeakerLegal : (1u << actions_of(kScen)) - 1u;
+}
+
+// One thread, one step: the agents whose bits from 16 on are set in act_pk (their
+// operands' parts were not finite somewhere) take their actions from a forward in fp32
+// FMAs of their observations, which are in the trajectory; ix: the step's agent 0.
+template <int N, int IN, int kScen, bool kLogits>
+__device__ __noinline__ uint32_t redo_agents(const RolloutArgs& a, int pair, int64_t ix, uint64_t g, uint32_t t,
+                                             uint32_t act_pk) {
+    constexpr int A = actions_of(kScen), XS = MlpX3<IN, A>::XS;
+    for (int i = 0; i < N; ++i) {
+        if (((act_pk >> (16 + i)) & 1u) == 0u) continue;
+        float z[A];
+        forward_fma<IN, MlpX3<IN, A>::H, A>(a.arena + a.pol_offset[a.pairs[pair * N + i]], a.obs + (ix + i) * XS, z);
+        const float uu = u24(draw(g, t, (uint32_t)i, a.seed).x);
+        act_pk = (act_pk & ~(0xfu << (4 * i))) | (uint32_t)sample_masked<A>(z, legal_of<kScen>(i), uu) << (4 * i);
+        if (kLogits)
+            for (int k = 0; k < A; ++k) a.logits[(ix + i) * A + k] = z[k];
+    }
+    return act_pk;
+}
+
 // kLogits: the call records the logits (the recording code is compiled out of
 // the other instance). blockDim.x = 128 groups.
 template <int N, int IN, int kScen = kSpread, bool kLogits = false>
 __global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
-    spread_rollout_x3_kernel(RolloutArgs a, RolloutPlan plan) {
+    spread_rollout_x3_kernel(const __grid_constant__ RolloutArgs a, const __grid_constant__ RolloutPlan plan) {
     static_assert(kScen != kAdversary || (N == 3 && IN == kAdvObs), "the simple adversary has 3 agents, obs 14");
     static_assert(kScen != kSpeakerListener || (N == 2 && IN == kSlObs),
                   "the simple speaker listener has 2 agents, obs 11");
@@ -326,20 +351,15 @@ __global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
                     if (busy) {
                         float lg[A];
                         M::logits(tb, lane_q, pol, lg);
-                        if (mine && parts_failed(lg[0])) {
-                            // (its observation is in the trajectory since before layer 2)
-                            float z[A];
-                            forward_fma<IN, M::H, A>(a.arena + a.pol_offset[a.pairs[pair * N + i]], a.obs + (ix + i) * XS, z);
-#pragma unroll
-                            for (int k = 0; k < A; ++k) lg[k] = z[k];
-                        }
                         if (mine) {
-                            const unsigned legal = (kScen == kSpeakerListener && i == 0) ? kSlSpeakerLegal : (1u << A) - 1u;
-                            act_pk |= (uint32_t)sample_masked<A>(lg, legal, uu) << (4 * i);
+                            act_pk |= (uint32_t)sample_masked<A>(lg, legal_of<kScen>(i), uu) << (4 * i);
+                            if (parts_failed(lg[0])) act_pk |= 0x10000u << i;
                         }
                         if (kLogits) store_logits(i, lg);
                     }
                 }
+                // agents whose parts failed (a call in their own loop cost it 1 to 5 %)
+                if (act_pk >> 16 != 0u) act_pk = redo_agents<N, IN, kScen, kLogits>(a, pair, ix, g, (uint32_t)t, act_pk);
                 if (plan.share) {
                     // the other groups' actions (a buffer is written again only
                     // after the next exchange's barrier, be it in the next unit)
