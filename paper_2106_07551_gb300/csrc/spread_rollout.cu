@@ -359,7 +359,10 @@ __global__ void __launch_bounds__(kGroupThreads * kMaxGroups, 1)
                     }
                 }
                 // agents whose parts failed (a call in their own loop cost it 1 to 5 %)
-                if (act_pk >> 16 != 0u) act_pk = redo_agents<N, IN, kScen, kLogits>(a, pair, ix, g, (uint32_t)t, act_pk);
+                if (__any_sync(0xffffffffu, act_pk >> 16 != 0u)) {
+                    __syncwarp();                            // after the other lanes' stores of this row
+                    if (act_pk >> 16 != 0u) act_pk = redo_agents<N, IN, kScen, kLogits>(a, pair, ix, g, (uint32_t)t, act_pk);
+                }
                 if (plan.share) {
                     // the other groups' actions (a buffer is written again only
                     // after the next exchange's barrier, be it in the next unit)
