@@ -271,6 +271,19 @@ __device__ __forceinline__ void unpack_hand(uint32_t w, LeducHand& h, int& t) {
     h.payoff = 0;
 }
 
+// The logits of the hand w in fp32 FMAs (its operands' parts were not finite
+// somewhere), a function of its own to keep its registers out of the tiles' loop.
+template <int H>
+__device__ __noinline__ float3 redo_logits(const float* __restrict__ img, uint32_t w) {
+    LeducHand h;
+    int t;
+    unpack_hand(w, h, t);
+    float o[17], z[3];
+    leduc_obs(h, o);
+    forward_fma<17, H, 3>(img, o, z);
+    return make_float3(z[0], z[1], z[2]);
+}
+
 // Units of a call: n_seg segments of `per` hands per pair.
 struct LeducUnits {
     int64_t n_seg, per, n_units;
@@ -464,10 +477,8 @@ __global__ void __launch_bounds__(kThreads, 1) leduc_eval_x3_kernel(EvalArgs a, 
                         int t;
                         unpack_hand(w, h, t);
                         if (parts_failed(lg[0])) {
-                            float ob[17], z[3];
-                            leduc_obs(h, ob);
-                            forward_fma<17, H, 3>(a.arena + a.pol_offset[pol], ob, z);
-                            lg[0] = z[0]; lg[1] = z[1]; lg[2] = z[2];
+                            const float3 z = redo_logits<H>(a.arena + a.pol_offset[pol], w);
+                            lg[0] = z.x; lg[1] = z.y; lg[2] = z.z;
                         }
                         const int act = sample_masked<3>(lg, leduc_legal(h), u);
                         const int64_t e = e_lo + id;
