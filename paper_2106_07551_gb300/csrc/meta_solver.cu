@@ -13,6 +13,7 @@
 
 #include "internal.h"
 #include "malib.h"
+#include "quotient.cuh"
 
 namespace malib {
 
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
     extern __shared__ double smem_tab[];
     __shared__ double offered[2][kLpMaxDim + 1];             // [parity] this CTA's best entering column
     __shared__ __align__(16) Offer offers[2][kLpMaxCluster]; // [parity][CTA]
-    __shared__ double colq[kLpMaxDim + 1], prow[kLpMaxDim + 1];
+    __shared__ double colq[kLpMaxDim + 1], invs[kLpMaxDim], prow[kLpMaxDim + 1];
     __shared__ int basis[kLpMaxDim], label[kLpMaxDim];       // label: variable of each own column
     __shared__ Cand red[2][kLpWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -405,8 +406,7 @@ __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
             const int q = ce.i;
             const int q_col = q_rank == rank ? oc : -1;      // its column here, when this CTA owns it
             // leaving row: minimum ratio (ratios are >= 0), ties to the lowest
-            // basic index; the candidate index packs (basic index, row). A division:
-            // times a rounded reciprocal, 49 / 49 and 1 / 1 would not tie
+            // basic index; the candidate index packs (basic index, row)
             Cand cl = none;
             for (int r = tid; r <= m; r += kLpThreads) {
                 double a;
@@ -418,7 +418,11 @@ __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
                 else
                     a = Tb[(int64_t)oc * hs + r];
                 colq[r] = a;
-                if (r < m && a > eps) cl = pick(cl, Cand{-okey(Tb[(int64_t)w * hs + r] / a), basis[r] * 1024 + r});
+                if (r < m && a > eps) {
+                    const double inv = 1.0 / a;
+                    invs[r] = inv;
+                    cl = pick(cl, Cand{-okey(quotient(Tb[(int64_t)w * hs + r], a, inv)), basis[r] * 1024 + r});
+                }
             }
             cl = cta_best(cl);
             if (cl.k == kNone) break;                        // unbounded: cannot happen with B > 0
@@ -426,10 +430,8 @@ __global__ void __launch_bounds__(kLpThreads) lp_nash_kernel(
             degenerate = (okey_inv(-cl.k) == 0.0) ? degenerate + 1 : 0;
             if (degenerate > 2 * (m + n)) bland = true;
             // pivot on (p, q): the scaled row p first
-            if (tid <= w) {                                  // (few warps: fp64 divisions are slow)
-                const double inv = 1.0 / colq[p];
-                for (int c = tid; c <= w; c += kLpThreads) prow[c] = c == q_col ? inv : Tb[(int64_t)c * hs + p] * inv;
-            }
+            const double inv = invs[p];
+            for (int c = tid; c <= w; c += kLpThreads) prow[c] = c == q_col ? inv : Tb[(int64_t)c * hs + p] * inv;
             const int leaving = basis[p];
             __syncthreads();
             if (tid == 0) {
