@@ -296,7 +296,7 @@ int malib_eval_payoff_ex(malib_ctx* ctx, const int32_t* pair_ids, int32_t n_pair
  * in which cudaMalloc/cudaFree would synchronise the device and stall other
  * streams. This call allocates nothing: it calls no cudaMalloc, cudaFree or
  * allocating library routine. Its scratch (per-pair payoff sums, a decision
- * counter and per-pair hand counters) is a fixed file-scope device array of
+ * counter and a counter per pair) is a fixed file-scope device array of
  * 192 KiB + 8 B that every GPU loading the library holds until the process
  * exits.
  *  - pair_ids and payoff_out must be DEVICE buffers of the context's device

@@ -67,7 +67,7 @@ struct EvalArgs {
     uint64_t seed;
     unsigned long long* acc;     // [n_pairs][2]
     unsigned long long* n_dec;   // total decisions (env-steps) of the call
-    unsigned long long* work;    // [n_pairs] hands claimed so far (zeroed per call)
+    unsigned long long* work;    // [n_pairs]: Leduc, units claimed so far (the first); Kuhn, a pair's blocks or decisions
     double* fin_out;             // Kuhn: [n_pairs][4] table written by each pair's last
                                  // block (work[] counts its finished blocks); null: a
                                  // separate finalize launch writes it

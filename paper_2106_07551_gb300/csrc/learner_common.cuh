@@ -42,7 +42,7 @@ __device__ __forceinline__ int64_t share_lo(const LearnArgs& a, int64_t c) {
 
 // Observation widths up to this one take the tensor-core kernel (learner_x3.cu): the
 // next one's two X tiles and W1 images would not fit its shared memory. 18 wide it
-// takes 1.08 ms where the general kernel takes 2.92; both take the same ReLU branches.
+// takes 1.08 ms where the general kernel takes 2.92; nearly all ReLU branches are the same.
 constexpr int kLearnX3MaxIn = 20;
 cudaError_t launch_learn_grad_x3(const LearnArgs& a, cudaStream_t s);
 

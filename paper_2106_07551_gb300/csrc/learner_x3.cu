@@ -507,9 +507,11 @@ __global__ void __launch_bounds__(kThreads, 1) learn_grad_x3_kernel(LearnArgs a)
 
     // A ReLU whose input is within rounding of zero may go either way, and each such
     // sample moves the gradient (a mean of terms of both signs) by ~1e-4 of its norm:
-    // inputs below 2^-20 of the row's others (13 times the difference of two fp32
-    // sums) take the sign of the fp32 chain, so that both kernels take the same
-    // branches. About one tile in 50 has such an input.
+    // inputs below 2^-20 of the largest of eight of the row's (13 times the usual
+    // difference of two fp32 sums) take the sign of the fp32 chain, so that nearly
+    // always both kernels take the same branch. Not always: the sums' difference goes
+    // with their terms, and a unit whose terms cancel far below them can differ by more.
+    // About one tile in 50 has an input this close to zero.
     auto settle = [&](float (&z)[32], int layer, int odd) {
         float mn = fabsf(z[0]), mx = mn;
 #pragma unroll

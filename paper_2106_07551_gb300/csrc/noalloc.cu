@@ -10,14 +10,16 @@
 // scratch (the per-pair payoff sums and the decision counter) lives in the
 // file-scope device array below instead of context-owned memory grown with
 // cudaMallocAsync, and it stages nothing (pair table and output must already
-// be device buffers). The scratch also holds the per-pair hand counters from
-// which the fp32 Leduc kernel's CTAs claim work units.
+// be device buffers). The scratch also holds a word per pair: the first is the
+// counter from which the fp32 Leduc kernel's CTAs claim work units; Kuhn's count
+// a pair's blocks, or its decisions.
 //
 // The array has room for kNoAllocMaxPairs pairs: (3 * 8192 + 1) x 8 bytes
-// (sums, decision counter, hand counters), 192 KiB + 8 B, held by every GPU
-// that loads the library until the process exits. Every call shares it and it keeps the previous call's contents, so
-// each call clears it first; calls that overlap on the GPU (two streams, or two
-// contexts on one device) race on it and must be serialised by the caller.
+// (sums, decision counter, a word per pair), 192 KiB + 8 B, held by every GPU
+// that loads the library until the process exits. Every call shares it, and it
+// keeps the previous call's contents, so each call clears what it adds to; calls
+// that overlap on the GPU (two streams, or two contexts on one device) race on it
+// and must be serialised by the caller.
 #include <cstdint>
 #include <mutex>
 

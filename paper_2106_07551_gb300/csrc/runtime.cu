@@ -646,7 +646,7 @@ int malib_eval_payoff_ex(malib_ctx* c, const int32_t* pair_ids, int32_t n_pairs,
         time_end(c, e0, e1);
         c->launches += 1;
     } else {
-        // [n_pairs][2] sums, the decision count, [n_pairs] hand-claim counters
+        // [n_pairs][2] sums, the decision count, [n_pairs] words (EvalArgs::work)
         if ((r = ensure(c, c->acc, c->acc_cap, (int64_t)n_pairs * 3 + 1, "payoff sums")) != MALIB_OK)
             return r;
         a.acc = c->acc;
