@@ -39,11 +39,13 @@
 //
 // What bounds it (17-128-128-3): layer 2's 98 MMAs of N = 64 take 1,620 cycles per
 // 64 output units, near the pipe's rate; on 64 x 65,536 hands the tensor pipe is
-// 59 % busy (two groups overlap), and a phase costs about 4,000 cycles of policy
+// 62 % busy (two groups overlap), and a phase costs about 4,000 cycles of policy
 // conversion and 7,800 of its first tile's chain, which is all there is in small
 // calls. 64 pairs x 65,536 hands: 12.24 ms with packed fp32 FMAs on 248 hands in
-// flight per CTA (0.64 of the FMA pipe), now 2.62 ms; 18 pairs x 338 hands: 237
-// us, now 74. The logits are off by 1.44e-7 of their norm against 64 bits (FMAs:
+// flight per CTA (0.64 of the FMA pipe), now 2.64 ms; 18 pairs x 338 hands: 237
+// us, now 74. 64 wide, many pairs of few hands are units' fixed costs: 4,900 pairs x
+// 20 hands 757 us before, 740 with both policies resident (832 converting in every
+// phase). The logits are off by 1.44e-7 of their norm against 64 bits (FMAs:
 // 1.73e-7; H = 64: 1.02e-7, before 1.18e-7).
 #include "device_common.cuh"
 #include "eval_common.cuh"

@@ -269,9 +269,9 @@ __global__ void __launch_bounds__(32 * W) aggregate_kernel(
 // the others read), one cluster barrier decides, and the ratio test and the
 // update run in every CTA without further exchange. The column buffer is
 // selected by the pivot's parity, so it is written again only after the next
-// barrier. One 100 x 100 game: 186 us on 8 CTAs (about 100 pivots); the full
-// tableau (identity columns included, a division per element to find its row) on
-// one CTA 780.
+// barrier. One 100 x 100 game (its pivots depend on its entries): 298 us on 8 CTAs
+// where the full tableau (identity columns included, a division per element to find
+// its row) on one CTA takes 1,237.
 // ---------------------------------------------------------------------------
 constexpr int kLpThreads = 256, kLpWarps = kLpThreads / 32;
 constexpr int kLpMaxDim = 512, kLpMaxCluster = 8;

@@ -85,8 +85,8 @@ def test_small_and_ragged(orc, n_eps):
 
 @pytest.mark.parametrize("n_eps", [3, 1000])
 def test_claimed_hands_across_pairs(orc, n_eps):
-    """64 pairs: with 3 hands per pair one CTA walks every pair; with 1,000 more
-    CTAs than pairs share each pair's hands. Every hand is replayed."""
+    """64 pairs: with 3 hands per pair a unit is a pair; with 1,000 the CTAs claim more
+    units than pairs. Every hand is replayed."""
     need_gpu()
     w = workloads.leduc(pop=8, hidden=128, with_bias=True, seed=77)
     ctx = context()
